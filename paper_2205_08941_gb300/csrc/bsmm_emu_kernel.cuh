@@ -32,6 +32,8 @@
 // Every wait is bounded as in the split kernel; a CTA that gives up retires its copies and
 // MMAs, frees its tensor memory and sets bit 16 of the context flag.
 constexpr int NSE = 4;                       // shared-memory stages (one K step each)
+constexpr int E_ST = 320;                    // threads per CTA (10 warps)
+constexpr int E_PROD = 0, E_MMA = 1;         // producer warp, MMA warp
 constexpr int E_AMAIN = EMU_P * COLB_A;      // 16 KB: an A main piece (planes x one column)
 constexpr int E_BMAIN = EMU_P * COLB_B;      // 8 KB
 constexpr int E_ATAIL = 2 * E_AMAIN;         // 32 KB: an A tail piece (planes x two columns)
@@ -142,7 +144,7 @@ __device__ __forceinline__ void tm_st8(uint32_t addr, const uint32_t (&v)[8])
 }
 
 template <int NB>
-__global__ void __launch_bounds__(ST, 1) k_bsmm_emu(const EmuArgs p)
+__global__ void __launch_bounds__(E_ST, 1) k_bsmm_emu(const EmuArgs p)
 {
     constexpr int GI = MT / NB, GJ = NT / NB;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_emu(const EmuArgs p)
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == W_MMA) {
+    if (warp == E_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&bars->tmem_slot)),
                      "r"(E_TMEM_COLS));
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_emu(const EmuArgs p)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = bars->tmem_slot;
 
-    if (warp == W_PROD) {
+    if (warp == E_PROD) {
         // ------------------------------------------------------------ producer
         uint32_t sg = 0;  // running stage (K step) counter
         int last[NSE];
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_emu(const EmuArgs p)
                 if (last[s] >= 0 && !bar_wait_plain(smem_u32(&bars->full[s]), (last[s] / NSE) & 1))
                     *abort_flag = 1;
         __syncwarp();
-    } else if (warp == W_MMA) {
+    } else if (warp == E_MMA) {
         // ------------------------------------------------------------ MMA issue
         // the warp walks the K steps (its lanes load the period flags 32 steps at a time);
         // lane 0 waits and issues
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_emu(const EmuArgs p)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (t == 0 && *abort_flag) atomicOr(p.flag, 16);
-    if (warp == W_MMA) {
+    if (warp == E_MMA) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(E_TMEM_COLS));

@@ -51,13 +51,12 @@
 
 namespace {
 
-constexpr int ST = 320;                      // threads per CTA (10 warps)
 constexpr int MT = 128, NT = 64, KCH = 48;   // tile M, N and K chunk
 constexpr int KSTEPS = KCH / 16;             // MMA K steps per chunk
 constexpr int A_CHUNK = 3 * MT * KCH * 2;   // 36 KB: three planes of 128 rows x 48 K
 constexpr int B_CHUNK = 3 * NT * KCH * 2;   // 18 KB
 constexpr int STAGE = A_CHUNK + B_CHUNK;    // one shared-memory stage of the split kernel
-constexpr int BAR_BYTES = 256;
+constexpr int BAR_BYTES = 512;
 constexpr int DRAIN = 4;                     // chunks per FP32 accumulation period
 constexpr int NACC = 4;                      // FP32 accumulators in tensor memory
 constexpr int TMEM_COLS = NACC * NT;
@@ -417,6 +416,7 @@ struct SplitArgs {
     int c_stride;
     double alpha, beta;
     int32_t *flag;
+    uint32_t *counter;        // two zero words: tiles handed out, CTAs done (left at zero)
     long long test_wait_cycles;  // > 0: test mode, the MMA thread's first wait runs out
     // mixed basis only (bsmm_mixed.cuh): tiles of this launch, row tables, C block offsets
     const int2 *tiles;
@@ -1244,6 +1244,7 @@ cq_status run_split(cq_ctx *ctx, const PiecePlan *pl, const Groups *gr, double a
         a.alpha = alpha;
         a.beta = beta;
         a.flag = ctx->flag.as<int32_t>();
+        a.counter = ctx->flag.as<uint32_t>() + 1;  // words 1 and 2 of the flag buffer
         a.test_wait_cycles = ctx->test_wait_cycles;
         a.tiles = pl->tiles.as<int2>() + b.tile0;
         a.g_row = gr->g_row.as<int32_t>();
@@ -1375,7 +1376,7 @@ cq_status run_emu(cq_ctx *ctx, PiecePlan *pl, const Groups *gr, double alpha,
             pl->n_steps > 0 ? (double)pl->batch_steps[q] / (double)pl->n_steps : 0.0;
         const int grid = std::min(a.n_tiles, ctx->num_sms);
         cq_timing_begin(ctx, flops * share, pl->mma_flops * share);
-        k_bsmm_emu<NB><<<grid, ST, SMEM_E, s>>>(a);
+        k_bsmm_emu<NB><<<grid, E_ST, SMEM_E, s>>>(a);
         cq_timing_end(ctx);
         cq_count_launch();
         if ((st = cq_check_cuda(ctx, cudaGetLastError(), "bsmm_emu")) != CQ_OK) return st;

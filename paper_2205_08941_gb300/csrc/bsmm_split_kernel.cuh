@@ -1,31 +1,60 @@
 // The tile kernel of the split-BF16 product (included by bsmm_split.cu).
 //
-// Warp roles (10 warps, one CTA per SM):
-//   warp 0      producer: a chunk is up to three consecutive K steps of a tile; lane 0
-//               copies each K step's pieces (main step: two A and two B main pieces; tail
-//               step: one A and one B tail piece; 18 KB either way) into the step's slot of
-//               a free stage with TMA bulk copies that complete on the stage's "full"
-//               barrier; the warp's lanes load the K-step table 32 entries at a time;
-//   warp 1      lane 0 issues the MMAs of a chunk (6 split products per K step) into
-//               one of NACC TMEM accumulators (one per drain period, in rotation) and
-//               commits them to the stage's "empty" barrier, and at the end of a drain
-//               period to the accumulator's "full" barrier;
-//   warps 2-9   drain: every DRAIN chunks they read the FP32 accumulator (warp w: TMEM lane
-//               quarter w % 4, columns 32 * ((w - 2) / 4) ..) into double-float (hi, lo)
-//               sums in registers, release the accumulator, and write C after a tile's last
-//               period.
+// Warp roles (12 warps, one CTA per SM):
+//   warps 0-7   drain: every DRAIN chunks they read the FP32 accumulator (warp w: TMEM lane
+//               quarter w % 4, columns 32 * (w / 4) ..) into double-float (hi, lo) sums in
+//               registers, release the accumulator, and write C after a tile's last period;
+//   warps 8, 9  producers of the A and of the B pieces: a chunk is up to three consecutive K
+//               steps of a tile; its pieces (main step: two A and two B main pieces; tail step:
+//               one A and one B tail piece; 18 KB either way) go into the step's slot of a
+//               free stage with TMA bulk copies that complete on the stage's "full" barrier;
+//   warp 10     one elected lane issues the MMAs of a chunk (6 split products per K step)
+//               into one of NACC TMEM accumulators (one per drain period, in rotation) and
+//               commits them to the stage's "empty" barrier, and at the end of a drain period
+//               to the accumulator's "full" barrier;
+//   warp 11     scheduler: takes the launch's next tile from a global counter and queues it for
+//               the other warps (NTQ tiles ahead).
 // Stages rotate over one running chunk counter across all tiles of the CTA; accumulators
 // over one running period counter; every wait computes its parity from those counters.
+//
+// What bounds it, on the 4096-atom SZP cell's U.X kept on P_L (25.7 M K steps of 169 K per
+// SM, 18 KB each): first the issue of copies and MMAs from single-lane branches, then HBM.
+//  * A bulk copy costs its issuing thread 70-126 clocks whatever its size (one warp: 1291
+//    clocks for the 12 copies of a chunk; two warps work side by side), so two producer
+//    warps share a chunk, and pieces that are neighbours in memory move in one copy.
+//  * tcgen05.mma (N = 64) issues at 68 clocks from a single-lane branch with descriptors in
+//    ordinary registers, at 58 from warp-uniform code with an elected lane; the operands
+//    alone take 48 (6 KB of shared memory at 128 B per clock).
+//  * With tiles dealt round-robin the CTAs drifted apart until the tiles in flight spanned
+//    ten M groups: 345 GB of DRAM reads, 7.2 TB/s.  The queue keeps them neighbours, and the
+//    B pieces (read once per tile) are evicted first, so the A pieces of one or two M groups
+//    (9 MB each) stay in L2.
+// Measured on that product: 316 ns per K step and SM before (53.5 ms with two producers in
+// place of one, 60.8 ms as it was), 282 with warp-uniform issue, 253 with the eviction
+// policies, 204 with the queue (34.6 ms).  The MMAs' own limit is 178 ns.
 //
 // Every wait is bounded (about two seconds) and also ends when another role has given up:
 // the CTA then stops issuing work, retires its own copies and MMAs (bounded), frees its
 // tensor memory and returns with bit 16 of the context flag set.
 constexpr int NS = 4;                  // shared-memory stages
 constexpr int N_DRAIN = 256;           // drain threads
-constexpr int W_PROD = 0, W_MMA = 1;   // producer warp, MMA warp
+constexpr int NPROD = 2;               // producer warps
+constexpr int W_PROD = 8, W_MMA = W_PROD + NPROD;  // first producer warp, MMA warp (0-7 drain)
+constexpr int W_SCHED = W_MMA + 1;     // scheduler warp
+constexpr int ST = 32 * (W_SCHED + 1); // threads per CTA (12 warps)
+constexpr int NTQ = 2;                 // tiles queued ahead
+constexpr int TILE_READERS = NPROD + 1 + N_DRAIN / 32;  // warps that read each queued tile
+
+// A queued tile: its index, first K step, K steps and main K steps (tile < 0: no more tiles)
+struct TileRec {
+    int64_t s0;
+    int32_t tile, nks, nm;
+};
 
 struct Bars {
     uint64_t full[NS], empty[NS], acc_full[NACC], acc_empty[NACC], done;
+    uint64_t tile_full[NTQ], tile_empty[NTQ];
+    TileRec rec[NTQ];
     uint64_t never;  // no thread ever arrives here: the test-only wait on it must run out
     uint32_t tmem_slot;
     int abort_flag;
@@ -46,9 +75,15 @@ __device__ __forceinline__ bool bar_try(uint32_t addr, uint32_t parity)
     return done != 0;
 }
 
+__device__ __forceinline__ void bar_arrive(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
 // Bounded wait on an mbarrier phase; gives up when another role has set the abort flag.
 __device__ __forceinline__ bool bar_wait(uint32_t addr, uint32_t parity, volatile int *abort_flag)
 {
+    if (bar_try(addr, parity)) return true;
     const long long t0 = clock64();
     while (!bar_try(addr, parity)) {
         if (*abort_flag) return false;
@@ -58,6 +93,37 @@ __device__ __forceinline__ bool bar_wait(uint32_t addr, uint32_t parity, volatil
         }
     }
     return true;
+}
+
+// bar_wait by a whole warp: its lanes go on together or give up together
+__device__ __forceinline__ bool warp_wait(uint32_t addr, uint32_t parity, volatile int *abort_flag)
+{
+    return __all_sync(0xffffffffu, bar_wait(addr, parity, abort_flag));
+}
+
+// bar_wait by lane 0 alone, its outcome for the whole warp
+__device__ __forceinline__ bool warp_wait_lane0(bool need, uint32_t addr, uint32_t parity,
+                                                volatile int *abort_flag, int lane)
+{
+    int go = 1;
+    if (need && lane == 0) go = bar_wait(addr, parity, abort_flag);
+    return __shfl_sync(0xffffffffu, go, 0) != 0;
+}
+
+// The n-th tile of this CTA from the queue, read by a whole warp (tile -1: none, or given up)
+__device__ __forceinline__ TileRec next_tile(Bars *bars, uint32_t n, volatile int *abort_flag,
+                                             int lane)
+{
+    TileRec r;
+    r.tile = -1;
+    r.s0 = 0;
+    r.nks = r.nm = 0;
+    if (warp_wait(smem_u32(&bars->tile_full[n % NTQ]), (n / NTQ) & 1u, abort_flag)) {
+        r = bars->rec[n % NTQ];
+        __syncwarp();
+        if (lane == 0) bar_arrive(smem_u32(&bars->tile_empty[n % NTQ]));
+    }
+    return r;
 }
 
 // Bounded wait with its own limit in cycles (the test-only short wait).
@@ -84,9 +150,11 @@ __device__ __forceinline__ bool bar_wait_plain(uint32_t addr, uint32_t parity)
     return true;
 }
 
-__device__ __forceinline__ void bar_arrive(uint32_t addr)
+__device__ __forceinline__ bool elect_one()
 {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr) : "memory");
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}\n" : "=r"(p));
+    return p != 0;
 }
 
 __device__ __forceinline__ void bar_commit(uint32_t addr)
@@ -105,6 +173,31 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
             dst),
         "l"(src), "r"(bytes), "r"(bar)
         : "memory");
+}
+
+// The same with an L2 eviction policy
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes,
+                                          uint32_t bar, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
+        "[%1], %2, [%3], %4;" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(bar), "l"(policy)
+        : "memory");
+}
+
+__device__ __forceinline__ uint64_t l2_evict_first()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+
+__device__ __forceinline__ uint64_t l2_evict_last()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    return p;
 }
 
 // Epilogue of one drain thread: accumulator row arow = (atom of M slot si, orbital a),
@@ -136,6 +229,98 @@ __device__ __forceinline__ void write_rows(const SplitArgs &p, const int32_t (&c
     }
 }
 
+// The six split products of one K step into the accumulator at acc_addr: a, b are the low
+// words of the step's plane-0 descriptors, PA and PB the plane strides in 16-byte units; acc
+// = 0 overwrites the accumulator.
+template <int PA, int PB>
+__device__ __forceinline__ void mma_step(uint32_t acc_addr, uint32_t a, uint32_t b, uint32_t acc)
+{
+    constexpr int pq[6][2] = {{0, 0}, {0, 1}, {1, 0}, {0, 2}, {1, 1}, {2, 0}};
+    constexpr uint32_t hi = (uint32_t)(128 >> 4) | (1u << 14);  // piece_desc's high word
+#pragma unroll
+    for (int x = 0; x < 6; ++x)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}\n" ::"r"(acc_addr),
+            "r"(a + pq[x][0] * PA), "r"(b + pq[x][1] * PB), "r"(IDESC), "r"(x == 0 ? acc : 1u), "r"(hi));
+}
+
+// One producer warp (SIDE 0: A pieces, 1: B pieces) over all chunks of the CTA's tiles.
+template <int SIDE>
+__device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *bars,
+                                        volatile int *abort_flag, int lane)
+{
+    constexpr int MAIN = SIDE ? B_MAIN : A_MAIN, TAIL = SIDE ? B_TAIL : A_TAIL;
+    constexpr int SLOT = SIDE ? B_SLOT : A_SLOT;
+    const uint8_t *mains = SIDE ? p.b_main : p.a_main - p.am0 * A_MAIN;
+    const uint8_t *tails = SIDE ? p.b_tail : p.a_tail - p.at0 * A_TAIL;
+    const uint32_t dst0 = sm0 + (SIDE ? B_SLOTS : 0) + lane * SLOT;
+    static_assert(TAIL == 2 * MAIN, "a tail piece fills a step's slot like two main pieces");
+    // K steps come PB at a time, one per lane, loaded one batch ahead (the next tile's first
+    // batch during this tile's last)
+    constexpr int PB = 32 / KSTEPS * KSTEPS;
+    auto load = [&](const TileRec &t, int base) {
+        return lane < PB && base + lane < t.nks
+                   ? __ldg(reinterpret_cast<const int2 *>(p.steps + t.s0 + base + lane) + SIDE)
+                   : make_int2(0, 0);
+    };
+    const uint64_t policy = SIDE ? l2_evict_first() : l2_evict_last();
+    uint32_t cg = 0;  // running chunk counter
+    bool ok = true;
+    TileRec t = next_tile(bars, 0, abort_flag, lane);
+    int2 cur = load(t, 0);
+    for (uint32_t n = 1; t.tile >= 0 && ok; ++n) {
+        TileRec tn = t;
+        for (int base = 0; base == 0 || base < t.nks; base += PB) {
+            int2 nxt;
+            if (base + PB < t.nks) {
+                nxt = load(t, base + PB);
+            } else {
+                tn = next_tile(bars, n, abort_flag, lane);
+                nxt = load(tn, 0);
+            }
+            for (int q0 = base; q0 < min(t.nks, base + PB); q0 += KSTEPS, ++cg) {
+                const uint32_t s = cg % NS, fb = smem_u32(&bars->full[s]);
+                const int ex = __shfl_sync(0xffffffffu, cur.x, q0 - base + lane);
+                const int ey = __shfl_sync(0xffffffffu, cur.y, q0 - base + lane);
+                if (!warp_wait_lane0(cg >= (uint32_t)NS, smem_u32(&bars->empty[s]),
+                                     ((cg / NS) + 1) & 1u, abort_flag, lane)) {
+                    ok = false;
+                    break;
+                }
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
+                                 "r"((uint32_t)(min(KSTEPS, t.nks - q0) * SLOT))
+                                 : "memory");
+                __syncwarp();
+                const int q = q0 + lane;
+                if (lane < KSTEPS && q < t.nks) {
+                    const uint32_t dst = dst0 + s * STAGE;
+                    const bool tail = q >= t.nm, pair = ey == ex + 1;
+                    bulk_copy(dst, tail ? tails + (int64_t)ex * TAIL : mains + (int64_t)ex * MAIN,
+                              tail || pair ? 2 * MAIN : MAIN, fb, policy);
+                    if (!tail && !pair)
+                        bulk_copy(dst + MAIN, ey < 0 ? p.zero : mains + (int64_t)ey * MAIN, MAIN, fb,
+                                  policy);
+                }
+            }
+            if (!ok) break;
+            cur = nxt;
+        }
+        t = tn;
+    }
+    // every copy lands before the CTA's shared memory is released.  A stage's barrier needs
+    // both sides: they arm the same chunks, since a free stage is seen by both (the barrier
+    // is tried before the abort flag)
+    if (lane == 0)
+        for (uint32_t k = 0; k < (uint32_t)NS && k < cg; ++k) {
+            const uint32_t c = cg - 1 - k;
+            if (!bar_wait_plain(smem_u32(&bars->full[c % NS]), (c / NS) & 1u)) *abort_flag = 1;
+        }
+    __syncwarp();
+}
+
 // NB = 0: mixed basis (groups, rows and columns through the tables of bsmm_mixed.cuh)
 template <int NB>
 __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
@@ -144,13 +329,13 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
     extern __shared__ __align__(1024) uint8_t smem[];
     Bars *bars = reinterpret_cast<Bars *>(smem + NS * STAGE);
     volatile int *abort_flag = &bars->abort_flag;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
     const uint32_t sm0 = smem_u32(smem);
 
     if (t == 0) {
         for (int s = 0; s < NS; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->full[s])),
-                         "r"(1));
+                         "r"(NPROD));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->empty[s])),
                          "r"(1));
         }
@@ -161,6 +346,12 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(
                              smem_u32(&bars->acc_empty[b])),
                          "r"(N_DRAIN));
+        }
+        for (int r = 0; r < NTQ; ++r) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->tile_full[r])),
+                         "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->tile_empty[r])),
+                         "r"(TILE_READERS));
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->done)), "r"(1));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->never)), "r"(1));
@@ -179,158 +370,132 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = bars->tmem_slot;
 
-    if (warp == W_PROD) {
-        // ------------------------------------------------------------ producer
-        uint32_t cg = 0;  // running chunk counter
-        int last[NS];     // last chunk issued into each stage (lane 0)
-#pragma unroll
-        for (int s = 0; s < NS; ++s) last[s] = -1;
+    if (warp == W_PROD || warp == W_PROD + 1) {
+        // ------------------------------------------------------------ producers
+        // warp W_PROD copies the A pieces of every chunk, the next warp the B pieces; lane x
+        // those of the chunk's K step x.  The two main pieces of a step are neighbours in
+        // memory when no atom of the group's list lies between the two, and then one copy
+        // moves both.
+        if (warp == W_PROD)
+            produce<0>(p, sm0, bars, abort_flag, lane);
+        else
+            produce<1>(p, sm0, bars, abort_flag, lane);
+    } else if (warp == W_MMA) {
+        // ------------------------------------------------------------ MMA issue
+        // the whole warp walks the chunks (uniform control flow keeps the descriptors in
+        // uniform registers: 58 clocks per MMA against 68 from a single-lane branch); one
+        // elected lane issues
+        const bool el = elect_one();
+        uint32_t cg = 0, pg = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-            const int64_t s0 = p.kstart[tile];
-            const int nks = (int)(p.kstart[tile + 1] - s0);
-            const int nm = p.nmain[tile];
-            const int nch = (nks + KSTEPS - 1) / KSTEPS;
-            int4 ent = make_int4(0, 0, 0, 0);
-            for (int c = 0; c < nch; ++c, ++cg) {
-                const int s = (int)(cg % NS);
-                const int nv = min(KSTEPS, nks - KSTEPS * c);  // K steps of this chunk
-                int go = 1;
-                if (lane == 0) {
-                    if (cg >= (uint32_t)NS &&
-                        !bar_wait(smem_u32(&bars->empty[s]), ((cg / NS) + 1) & 1u, abort_flag)) {
-                        go = 0;
-                    } else {
-                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-                                         smem_u32(&bars->full[s])),
-                                     "r"((uint32_t)(nv * (A_SLOT + B_SLOT)))
-                                     : "memory");
-                        last[s] = (int)cg;
-                    }
-                }
-                if (!__shfl_sync(0xffffffffu, go, 0)) {
+        // test mode: the first wait is on a barrier nothing completes, with a short limit,
+        // so it runs out; the CTA then takes the same abort path as a real timeout
+        if (p.test_wait_cycles > 0) {
+            bar_wait_for(smem_u32(&bars->never), 0u, abort_flag, p.test_wait_cycles);
+            ok = false;
+        }
+        // low words of the descriptors of slot 0 of stage 0 for both kinds of K step (main:
+        // the second column is the second atom's piece, A_MAIN / B_MAIN further; tail: the
+        // piece's second column); a stage, slot or plane only moves the 14-bit start address
+        // field (shared addresses stay below 256 KB, so no carry leaves it)
+        const uint32_t dam = (uint32_t)piece_desc(sm0, A_MAIN);
+        const uint32_t dat = (uint32_t)piece_desc(sm0, COLB_A);
+        const uint32_t dbm = (uint32_t)piece_desc(sm0 + B_SLOTS, B_MAIN);
+        const uint32_t dbt = (uint32_t)piece_desc(sm0 + B_SLOTS, COLB_B);
+        const uint32_t bar0 = smem_u32(bars);
+        for (uint32_t n = 0; ok; ++n) {
+            const TileRec tr = next_tile(bars, n, abort_flag, lane);
+            if (tr.tile < 0) break;
+            const int nks = tr.nks, nm = tr.nm;
+            int period = 0;  // chunks of the current drain period already issued
+            for (int q0 = 0; q0 < nks; q0 += KSTEPS, ++cg) {
+                const uint32_t b = pg % NACC;
+                if (period == 0 && pg >= (uint32_t)NACC &&
+                    !warp_wait(bar0 + (uint32_t)offsetof(Bars, acc_empty) + 8 * b,
+                               ((pg / NACC) + 1) & 1u, abort_flag)) {
                     ok = false;
                     break;
                 }
-                for (int x = 0; x < nv; ++x) {
-                    const int q = KSTEPS * c + x;
-                    if ((q & 31) == 0)
-                        ent = q + lane < nks ? p.steps[s0 + q + lane] : make_int4(0, 0, 0, 0);
-                    const int ea = __shfl_sync(0xffffffffu, ent.x, q & 31);
-                    const int ea2 = __shfl_sync(0xffffffffu, ent.y, q & 31);
-                    const int eb = __shfl_sync(0xffffffffu, ent.z, q & 31);
-                    const int eb2 = __shfl_sync(0xffffffffu, ent.w, q & 31);
-                    if (lane == 0) {
-                        const uint32_t fb = smem_u32(&bars->full[s]);
-                        const uint32_t da = sm0 + s * STAGE + x * A_SLOT;
-                        const uint32_t db = sm0 + s * STAGE + B_SLOTS + x * B_SLOT;
-                        if (q < nm) {
-                            bulk_copy(da, p.a_main + (int64_t)(ea - p.am0) * A_MAIN, A_MAIN, fb);
-                            bulk_copy(da + A_MAIN,
-                                      ea2 < 0 ? p.zero : p.a_main + (int64_t)(ea2 - p.am0) * A_MAIN,
-                                      A_MAIN, fb);
-                            bulk_copy(db, p.b_main + (int64_t)eb * B_MAIN, B_MAIN, fb);
-                            bulk_copy(db + B_MAIN, eb2 < 0 ? p.zero : p.b_main + (int64_t)eb2 * B_MAIN,
-                                      B_MAIN, fb);
-                        } else {
-                            bulk_copy(da, p.a_tail + (int64_t)(ea - p.at0) * A_TAIL, A_TAIL, fb);
-                            bulk_copy(db, p.b_tail + (int64_t)eb * B_TAIL, B_TAIL, fb);
-                        }
-                    }
+                const uint32_t s = cg % NS;
+                if (!warp_wait(bar0 + (uint32_t)offsetof(Bars, full) + 8 * s, (cg / NS) & 1u,
+                               abort_flag)) {
+                    ok = false;
+                    break;
                 }
-            }
-        }
-        if (lane == 0)  // every copy lands before the CTA's shared memory is released
-            for (int s = 0; s < NS; ++s)
-                if (last[s] >= 0 && !bar_wait_plain(smem_u32(&bars->full[s]), (last[s] / NS) & 1))
-                    *abort_flag = 1;
-        __syncwarp();
-    } else if (warp == W_MMA) {
-        // ------------------------------------------------------------ MMA issue
-        if (lane == 0) {
-            uint32_t cg = 0, pg = 0;
-            bool ok = true, issued = false;
-            // test mode: the first wait is on a barrier nothing completes, with a short limit,
-            // so it runs out; the CTA then takes the same abort path as a real timeout
-            if (p.test_wait_cycles > 0) {
-                bar_wait_for(smem_u32(&bars->never), 0u, abort_flag, p.test_wait_cycles);
-                ok = false;
-            }
-            const int pq[6][2] = {{0, 0}, {0, 1}, {1, 0}, {0, 2}, {1, 1}, {2, 0}};
-            // descriptors of slot 0 of stage 0 for both kinds of K step (main: the second
-            // column is the second atom's piece, A_MAIN / B_MAIN further; tail: the piece's
-            // second column); a stage, slot or plane only moves the 14-bit start address
-            // field (shared addresses stay below 256 KB, so no carry leaves it)
-            const uint64_t dam = piece_desc(sm0, A_MAIN), dat = piece_desc(sm0, COLB_A);
-            const uint64_t dbm = piece_desc(sm0 + B_SLOTS, B_MAIN);
-            const uint64_t dbt = piece_desc(sm0 + B_SLOTS, COLB_B);
-            for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-                const int nks = (int)(p.kstart[tile + 1] - p.kstart[tile]);
-                const int nm = p.nmain[tile];
-                const int nch = (nks + KSTEPS - 1) / KSTEPS;
-                for (int c = 0; c < nch; ++c, ++cg) {
-                    const uint32_t b = pg % NACC;
-                    if (c % DRAIN == 0 && pg >= (uint32_t)NACC &&
-                        !bar_wait(smem_u32(&bars->acc_empty[b]), ((pg / NACC) + 1) & 1u,
-                                  abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    const int s = (int)(cg % NS);
-                    if (!bar_wait(smem_u32(&bars->full[s]), (cg / NS) & 1u, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t acc_addr = tmem + b * NT;
-                    const int nv = min(KSTEPS, nks - KSTEPS * c);
-                    for (int ks = 0; ks < nv; ++ks) {
-                        const bool main_step = KSTEPS * c + ks < nm;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t acc_addr = tmem + b * NT;
+                const bool last = q0 + KSTEPS >= nks || period == DRAIN - 1;
+                if (el) {
+#pragma unroll
+                    for (int ks = 0; ks < KSTEPS; ++ks) {
+                        if (q0 + ks >= nks) break;
+                        const uint32_t oa = s * (STAGE >> 4) + ks * (A_SLOT >> 4);
+                        const uint32_t ob = s * (STAGE >> 4) + ks * (B_SLOT >> 4);
+                        const uint32_t acc = period == 0 && ks == 0 ? 0u : 1u;
                         // plane strides in 16-byte units: main pieces hold one column per
                         // plane, tail pieces two
-                        const uint32_t pa = main_step ? COLB_A >> 4 : (2 * COLB_A) >> 4;
-                        const uint32_t pb = main_step ? COLB_B >> 4 : (2 * COLB_B) >> 4;
-                        const uint64_t sa = (main_step ? dam : dat) +
-                                            (uint64_t)((s * STAGE + ks * A_SLOT) >> 4);
-                        const uint64_t sb = (main_step ? dbm : dbt) +
-                                            (uint64_t)((s * STAGE + ks * B_SLOT) >> 4);
-#pragma unroll
-                        for (int x = 0; x < 6; ++x) {
-                            const uint64_t ad = sa + (uint64_t)(pq[x][0] * pa);
-                            const uint64_t bd = sb + (uint64_t)(pq[x][1] * pb);
-                            const uint32_t acc = (c % DRAIN == 0 && ks == 0 && x == 0) ? 0u : 1u;
-                            asm volatile(
-                                "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(
-                                    acc_addr),
-                                "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
-                        }
+                        if (q0 + ks < nm)
+                            mma_step<COLB_A / 16, COLB_B / 16>(acc_addr, dam + oa, dbm + ob, acc);
+                        else
+                            mma_step<2 * COLB_A / 16, 2 * COLB_B / 16>(acc_addr, dat + oa, dbt + ob, acc);
                     }
-                    bar_commit(smem_u32(&bars->empty[s]));
-                    issued = true;
-                    if (c % DRAIN == DRAIN - 1 || c == nch - 1) {
-                        bar_commit(smem_u32(&bars->acc_full[b]));
-                        ++pg;
-                    }
+                    bar_commit(bar0 + (uint32_t)offsetof(Bars, empty) + 8 * s);
+                    if (last) bar_commit(bar0 + (uint32_t)offsetof(Bars, acc_full) + 8 * b);
                 }
+                __syncwarp();
+                period = last ? 0 : period + 1;
+                pg += last;
             }
-            if (issued) {  // retire every MMA before the tensor memory is released
-                bar_commit(smem_u32(&bars->done));
-                if (!bar_wait_plain(smem_u32(&bars->done), 0u)) *abort_flag = 1;
+        }
+        // retire every MMA before the tensor memory is released
+        if (cg > 0 && el) {
+            bar_commit(smem_u32(&bars->done));
+            if (!bar_wait_plain(smem_u32(&bars->done), 0u)) *abort_flag = 1;
+        }
+        __syncwarp();
+    } else if (warp == W_SCHED) {
+        // ------------------------------------------------------------ scheduler
+        // hands out the launch's tiles in order, so that the tiles in flight on the GPU stay
+        // neighbours (they share the A pieces of one or two M groups) and no CTA idles while
+        // others hold several tiles
+        if (lane == 0) {
+            int i = blockIdx.x;
+            for (uint32_t n = 0;; ++n) {
+                TileRec r;
+                r.tile = -1;
+                r.s0 = 0;
+                r.nks = r.nm = 0;
+                if (i < p.n_tiles) {
+                    r.tile = i;
+                    r.s0 = p.kstart[r.tile];
+                    r.nks = (int)(p.kstart[r.tile + 1] - r.s0);
+                    r.nm = p.nmain[r.tile];
+                }
+                if (n >= (uint32_t)NTQ &&
+                    !bar_wait(smem_u32(&bars->tile_empty[n % NTQ]), ((n / NTQ) + 1) & 1u, abort_flag))
+                    break;
+                bars->rec[n % NTQ] = r;
+                bar_arrive(smem_u32(&bars->tile_full[n % NTQ]));
+                if (r.tile < 0) break;
+                i = (int)gridDim.x + (int)atomicAdd(&p.counter[0], 1u);
             }
+            // the last CTA to finish handing out resets the counters for the next launch
+            __threadfence();
+            if (atomicInc(&p.counter[1], gridDim.x - 1) == gridDim.x - 1) atomicExch(&p.counter[0], 0u);
         }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ drain and epilogue
-        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        const int quarter = warp & 3, half = warp >> 2;
         const int arow = quarter * 32 + lane;
         const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 32);
         uint32_t pg = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-            const int nks = (int)(p.kstart[tile + 1] - p.kstart[tile]);
-            const int nch = (nks + KSTEPS - 1) / KSTEPS;
-            const int np = (nch + DRAIN - 1) / DRAIN;
+        for (uint32_t n = 0; ok; ++n) {
+            const TileRec tr = next_tile(bars, n, abort_flag, lane);
+            if (tr.tile < 0) break;
+            const int tile = tr.tile;
+            const int np = (tr.nks + KSTEPS * DRAIN - 1) / (KSTEPS * DRAIN);
             // this row's C blocks, loaded now and used after the tile's last period
             constexpr int NJ = epi_slots<NB>();
             int32_t cid[NJ];
@@ -347,7 +512,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             for (int x = 0; x < 32; ++x) hi[x] = lo[x] = 0.f;
             for (int d = 0; d < np; ++d, ++pg) {
                 const uint32_t b = pg % NACC;
-                if (!bar_wait(smem_u32(&bars->acc_full[b]), (pg / NACC) & 1u, abort_flag)) {
+                if (!warp_wait(smem_u32(&bars->acc_full[b]), (pg / NACC) & 1u, abort_flag)) {
                     ok = false;
                     break;
                 }
