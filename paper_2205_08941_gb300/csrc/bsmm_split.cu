@@ -43,7 +43,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <numeric>
+#include <type_traits>
 
 #include "cq_internal.cuh"
 #include "emu_digits.cuh"
@@ -397,6 +399,18 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x)
     const float err = (hi - (s - bp)) + (x - bp);
     hi = s;
     lo += err;
+}
+
+// float -> double by its bits (a select for zeros, the conversion only for denormals,
+// infinities and NaNs): conversions to 64 bits run at the FP64 pipe's two lanes per clock and
+// SM, integer operations at 64 and more
+__device__ __forceinline__ double f32_to_f64(float x)
+{
+    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m - 1u >= 0x007fffffu && m < 0x7f800000u)  // zero or normal
+        return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u)),
+                                (int)(u << 29));
+    return (double)x;
 }
 
 struct SplitArgs {

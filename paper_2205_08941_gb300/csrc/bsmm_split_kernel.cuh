@@ -200,33 +200,78 @@ __device__ __forceinline__ uint64_t l2_evict_last()
     return p;
 }
 
+// Writes one row's columns of a block, values w[b] for b in [B0, B1) (b a column of the
+// block), at dst = the row's first column: 16-byte stores where two neighbours share one.
+// odd: whether dst is an odd multiple of eight bytes.
+template <int NB, int B0, int B1>
+__device__ __forceinline__ void put_row(double *dst, bool odd, const double (&w)[NB])
+{
+    constexpr int N = B1 - B0;
+    if constexpr (N <= 0) return;
+    const bool s = odd != (bool)(B0 & 1);  // a single value comes first
+#pragma unroll
+    for (int t = 0; t < (N - 1) / 2; ++t) {
+        const int b = B0 + 2 * t;
+        *reinterpret_cast<double2 *>(dst + b + s) =
+            make_double2(s ? w[b + 1] : w[b], s ? w[b + 2] : w[b + 1]);
+    }
+    if constexpr (N & 1) {
+        dst[s ? B0 : B1 - 1] = s ? w[B0] : w[B1 - 1];
+    } else if (!s) {
+        *reinterpret_cast<double2 *>(dst + B1 - 2) = make_double2(w[B1 - 2], w[B1 - 1]);
+    } else {
+        dst[B0] = w[B0];
+        dst[B1 - 1] = w[B1 - 1];
+    }
+}
+
 // Epilogue of one drain thread: accumulator row arow = (atom of M slot si, orbital a),
 // columns 32*HALF .. +31 = (atom of N slot, orbital); cid[u] is the P_C block of slot pair
-// (si, J0 + u) or -1; each present block gets beta*C + alpha*(hi + lo).
+// (si, J0 + u) or -1; each present block gets beta*C + alpha*v(column).  The plain case
+// (alpha 1, beta 0, C on a 16-byte boundary) costs one FP64 addition per value and stores 16
+// bytes at a time; the general one is bound by its four FP64-pipe operations per value.
 template <int NB> __host__ __device__ constexpr int epi_slots() { return 32 / (NB ? NB : 32) + 2; }
 
-template <int NB, int HALF>
-__device__ __forceinline__ void write_rows(const SplitArgs &p, const int32_t (&cid)[epi_slots<NB>()],
-                                           int arow, const float (&hi)[32], const float (&lo)[32])
+template <int NB, int HALF, class V>
+__device__ __forceinline__ void write_rows(double *C, int c_stride, double alpha, double beta,
+                                           const int32_t (&cid)[epi_slots<NB>()], int arow, V v)
 {
-    constexpr int GI = MT / NB, GJ = NT / NB;
-    constexpr int J0 = (HALF * 32) / NB, J1 = (HALF * 32 + 31) / NB;
+    constexpr int GI = MT / NB, GJ = NT / NB, H0 = HALF * 32;
+    constexpr int J0 = H0 / NB, J1 = (H0 + 31) / NB;
     if (arow >= GI * NB) return;
     const int a = arow % NB;
+    const bool plain = alpha == 1.0 && beta == 0.0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+    const bool odd = (a * NB) & 1;
+    auto block = [&](auto jc) {
+        constexpr int jl = J0 + decltype(jc)::value;
+        if constexpr (jl <= J1 && jl < GJ && jl - J0 < epi_slots<NB>()) {
+            const int32_t blk = cid[jl - J0];
+            if (blk < 0) return;
+            constexpr int B0 = jl * NB < H0 ? H0 - jl * NB : 0;
+            constexpr int B1 = (jl + 1) * NB > H0 + 32 ? H0 + 32 - jl * NB : NB;
+            double *dst = C + (int64_t)blk * c_stride + a * NB;
+            double w[NB];
 #pragma unroll
-    for (int jl = J0; jl <= J1; ++jl) {
-        if (jl >= GJ || jl - J0 >= epi_slots<NB>()) continue;
-        const int32_t blk = cid[jl - J0];
-        if (blk < 0) continue;
-        double *dst = p.C + (int64_t)blk * p.c_stride + a * NB;
+            for (int b = B0; b < B1; ++b) w[b] = v(jl * NB + b - H0);
+            if (plain) {
+                put_row<NB, B0, B1>(dst, odd, w);
+            } else {
 #pragma unroll
-        for (int bo = 0; bo < NB; ++bo) {
-            const int x = jl * NB + bo - HALF * 32;
-            if (x < 0 || x >= 32) continue;
-            const double v = (double)hi[x] + (double)lo[x];
-            dst[bo] = p.beta == 0.0 ? p.alpha * v : p.beta * dst[bo] + p.alpha * v;
+                for (int b = B0; b < B1; ++b)
+                    dst[b] = beta == 0.0 ? alpha * w[b] : beta * dst[b] + alpha * w[b];
+            }
         }
-    }
+    };
+    static_assert(J1 - J0 < 9, "slots of a half");
+    block(std::integral_constant<int, 0>());
+    block(std::integral_constant<int, 1>());
+    block(std::integral_constant<int, 2>());
+    block(std::integral_constant<int, 3>());
+    block(std::integral_constant<int, 4>());
+    block(std::integral_constant<int, 5>());
+    block(std::integral_constant<int, 6>());
+    block(std::integral_constant<int, 7>());
+    block(std::integral_constant<int, 8>());
 }
 
 // The six split products of one K step into the accumulator at acc_addr: a, b are the low
@@ -537,10 +582,11 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             }
             if (!ok) break;
             if constexpr (NB > 0) {
+                auto v = [&](int x) { return f32_to_f64(hi[x]) + f32_to_f64(lo[x]); };
                 if (half == 0)
-                    write_rows<NB, 0>(p, cid, arow, hi, lo);
+                    write_rows<NB, 0>(p.C, p.c_stride, p.alpha, p.beta, cid, arow, v);
                 else
-                    write_rows<NB, 1>(p, cid, arow, hi, lo);
+                    write_rows<NB, 1>(p.C, p.c_stride, p.alpha, p.beta, cid, arow, v);
             } else {
                 write_rows_mixed(p, tile, arow, half, hi, lo);
             }
