@@ -443,14 +443,14 @@ struct SplitArgs {
 #include "bsmm_emu_kernel.cuh"
 
 constexpr int SMEM = NS * STAGE + BAR_BYTES;     // pipeline stages + barriers
-constexpr int SMEM_E = NSE * E_STAGE + E_LWORDS + BAR_BYTES;
+constexpr int SMEM_E = NSE * E_STAGE + BAR_BYTES;
 
 // ---------------------------------------------------------------- emulated-FP64 plan and packing
 
 // K-step table of the emulated product (one thread per tile; COUNT writes the number of
 // steps of each tile, FILL the steps): per tail group the tile touches (ascending), main
 // steps pairing the tile's K atoms of that group (Morton ranks, ascending), then the group's
-// tail step; meta flags the first and the last (tail) step of each such scale period.
+// tail step, marked TAIL_STEP in its second entries, which ends the scale period.
 template <bool FILL>
 __global__ void __launch_bounds__(128)
 k_emu_steps(int n_tiles, int tg, const int2 *tiles, const int64_t *ka_start,
@@ -458,7 +458,7 @@ k_emu_steps(int n_tiles, int tg, const int2 *tiles, const int64_t *ka_start,
             const int64_t *gm_ptr, const int32_t *gm_key, const int64_t *hm_ptr,
             const int32_t *hm_key, const int64_t *gt_ptr, const int32_t *gt_key,
             const int64_t *ht_ptr, const int32_t *ht_key, const int64_t *step_start,
-            int64_t *count, int4 *steps, uint8_t *meta)
+            int64_t *count, int4 *steps)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= n_tiles) return;
@@ -479,12 +479,10 @@ k_emu_steps(int n_tiles, int tg, const int2 *tiles, const int64_t *ka_start,
             e.z = (int)list_pos(hm_key, hm_ptr[t.y], hm_ptr[t.y + 1], k0);
             e.w = k1 < 0 ? -1 : (int)list_pos(hm_key, hm_ptr[t.y], hm_ptr[t.y + 1], k1);
             steps[s] = e;
-            meta[s] = q == p ? PERIOD_FIRST : 0;
         }
         if (FILL) {
-            steps[s] = make_int4((int)list_pos(gt_key, gt_ptr[t.x], gt_ptr[t.x + 1], tau), -1,
-                                 (int)list_pos(ht_key, ht_ptr[t.y], ht_ptr[t.y + 1], tau), -1);
-            meta[s] = PERIOD_LAST | (p2 == p ? PERIOD_FIRST : 0);
+            steps[s] = make_int4((int)list_pos(gt_key, gt_ptr[t.x], gt_ptr[t.x + 1], tau), TAIL_STEP,
+                                 (int)list_pos(ht_key, ht_ptr[t.y], ht_ptr[t.y + 1], tau), TAIL_STEP);
         }
         ++s;
         p = p2;
@@ -580,7 +578,8 @@ k_pack_main_emu(int64_t e0, int64_t n, const int32_t *index, const int32_t *main
 }
 
 // Emulated tail pieces of entries [e0, e0 + n) (one thread per (entry, row)): as
-// k_pack_tail, eight digit planes against the row's group exponent.
+// k_pack_tail, eight digit planes against the row's group exponent, the second column's planes
+// after the first's (a tail piece reads like two main pieces).
 template <int NB, bool LEFT>
 __global__ void __launch_bounds__(256)
 k_pack_tail_emu(int64_t e0, int64_t n, const int32_t *index, const int16_t *scale,
@@ -609,7 +608,7 @@ k_pack_tail_emu(int64_t e0, int64_t n, const int32_t *index, const int16_t *scal
         emu_rows(x, 8, E, w);
 #pragma unroll
         for (int pl = 0; pl < EMU_P; ++pl)
-            *reinterpret_cast<uint4 *>(piece + piece_off(pl, 2 * COLB, c, COLB, r)) = w[pl];
+            *reinterpret_cast<uint4 *>(piece + piece_off(pl, COLB, c, EMU_P * COLB, r)) = w[pl];
     }
 }
 
@@ -652,15 +651,14 @@ struct PieceSet {
 
 // Plan of one tensor-core product (pattern triple): tiles, K-step table, batches.  Split
 // plans take the main steps of a tile first, then its tail steps; emulated plans take the
-// steps of one tail group (its scale period) together, its tail step last, and flag the
-// first and last step of every period in meta.
+// steps of one tail group (its scale period) together, its tail step last and marked.
 struct PiecePlan {
     int n_tiles = 0;
     int64_t n_steps = 0;
     double mma_flops = 0.0;  // tensor-core flops of one product over these tiles
     std::vector<PieceBatch> batches;
     std::vector<int64_t> batch_steps;
-    DevBuf tiles, kstart, nmain, steps, meta, cidx;
+    DevBuf tiles, kstart, nmain, steps, cidx;
     std::shared_ptr<PieceSet> ps;
 };
 
@@ -1109,7 +1107,7 @@ cq_status get_piece_plan(cq_ctx *ctx, int kind, const cq_pattern *pA, const cq_p
             pl->n_tiles, gr->tg, pl->tiles.as<int2>(), ka_start.as<int64_t>(),
             tile_rank.as<int32_t>(), kt_start.as<int64_t>(), tile_tau.as<int32_t>(), nullptr,
             nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-            cnt.as<int64_t>(), nullptr, nullptr);
+            cnt.as<int64_t>(), nullptr);
         cq_count_launch();
         std::vector<int64_t> c((size_t)pl->n_tiles);
         cudaMemcpyAsync(c.data(), cnt.ptr, 8 * c.size(), cudaMemcpyDeviceToHost, s);
@@ -1133,14 +1131,13 @@ cq_status get_piece_plan(cq_ctx *ctx, int kind, const cq_pattern *pA, const cq_p
             ps.bm.key.as<int32_t>(), ps.at.ptr.as<int64_t>(), ps.at.key.as<int32_t>(),
             ps.bt.ptr.as<int64_t>(), ps.bt.key.as<int32_t>(), pl->steps.as<int4>());
     } else {
-        if ((st = cq_alloc(ctx, pl->meta, (size_t)pl->n_steps + 16)) != CQ_OK) return st;
         k_emu_steps<true><<<(pl->n_tiles + 127) / 128, 128, 0, s>>>(
             pl->n_tiles, gr->tg, pl->tiles.as<int2>(), ka_start.as<int64_t>(),
             tile_rank.as<int32_t>(), kt_start.as<int64_t>(), tile_tau.as<int32_t>(),
             ps.am.ptr.as<int64_t>(), ps.am.key.as<int32_t>(), ps.bm.ptr.as<int64_t>(),
             ps.bm.key.as<int32_t>(), ps.at.ptr.as<int64_t>(), ps.at.key.as<int32_t>(),
             ps.bt.ptr.as<int64_t>(), ps.bt.key.as<int32_t>(), pl->kstart.as<int64_t>(), nullptr,
-            pl->steps.as<int4>(), pl->meta.as<uint8_t>());
+            pl->steps.as<int4>());
     }
     k_tile_cidx<<<pl->n_tiles, 256, 0, s>>>(
         pl->tiles.as<int2>(), gr->gi, gr->gj, gr->g_atoms.as<int32_t>(),
@@ -1370,7 +1367,6 @@ cq_status run_emu(cq_ctx *ctx, PiecePlan *pl, const Groups *gr, double alpha,
         a.n_tiles = b.tile1 - b.tile0;
         a.kstart = pl->kstart.as<int64_t>() + b.tile0;
         a.steps = pl->steps.as<int4>();
-        a.meta = pl->meta.as<uint8_t>();
         a.cidx = pl->cidx.as<int32_t>() + (int64_t)b.tile0 * gr->gi * gr->gj;
         a.a_main = (const uint8_t *)vam;
         a.am0 = b.am0;
@@ -1386,6 +1382,7 @@ cq_status run_emu(cq_ctx *ctx, PiecePlan *pl, const Groups *gr, double alpha,
         a.alpha = alpha;
         a.beta = beta;
         a.flag = ctx->flag.as<int32_t>();
+        a.counter = ctx->flag.as<uint32_t>() + 1;  // words 1 and 2 of the flag buffer
         const double share =
             pl->n_steps > 0 ? (double)pl->batch_steps[q] / (double)pl->n_steps : 0.0;
         const int grid = std::min(a.n_tiles, ctx->num_sms);

@@ -111,8 +111,8 @@ __device__ __forceinline__ bool warp_wait_lane0(bool need, uint32_t addr, uint32
 }
 
 // The n-th tile of this CTA from the queue, read by a whole warp (tile -1: none, or given up)
-__device__ __forceinline__ TileRec next_tile(Bars *bars, uint32_t n, volatile int *abort_flag,
-                                             int lane)
+template <class B>
+__device__ __forceinline__ TileRec next_tile(B *bars, uint32_t n, volatile int *abort_flag, int lane)
 {
     TileRec r;
     r.tile = -1;
@@ -226,29 +226,32 @@ __device__ __forceinline__ void put_row(double *dst, bool odd, const double (&w)
 }
 
 // Epilogue of one drain thread: accumulator row arow = (atom of M slot si, orbital a),
-// columns 32*HALF .. +31 = (atom of N slot, orbital); cid[u] is the P_C block of slot pair
-// (si, J0 + u) or -1; each present block gets beta*C + alpha*v(column).  The plain case
+// columns H0 .. H0 + W - 1 = (atom of N slot, orbital); cid[u] is the P_C block of slot pair
+// (si, H0 / NB + u) or -1; each present block gets beta*C + alpha*v(column).  The plain case
 // (alpha 1, beta 0, C on a 16-byte boundary) costs one FP64 addition per value and stores 16
 // bytes at a time; the general one is bound by its four FP64-pipe operations per value.
-template <int NB> __host__ __device__ constexpr int epi_slots() { return 32 / (NB ? NB : 32) + 2; }
-
-template <int NB, int HALF, class V>
-__device__ __forceinline__ void write_rows(double *C, int c_stride, double alpha, double beta,
-                                           const int32_t (&cid)[epi_slots<NB>()], int arow, V v)
+template <int NB, int W> __host__ __device__ constexpr int epi_slots()
 {
-    constexpr int GI = MT / NB, GJ = NT / NB, H0 = HALF * 32;
-    constexpr int J0 = H0 / NB, J1 = (H0 + 31) / NB;
+    return NB ? (W + NB - 2) / NB + 1 : 1;
+}
+
+template <int NB, int H0, int W, class V>
+__device__ __forceinline__ void write_rows(double *C, int c_stride, double alpha, double beta,
+                                           const int32_t (&cid)[epi_slots<NB, W>()], int arow, V v)
+{
+    constexpr int GI = MT / NB, GJ = NT / NB;
+    constexpr int J0 = H0 / NB, J1 = (H0 + W - 1) / NB;
     if (arow >= GI * NB) return;
     const int a = arow % NB;
     const bool plain = alpha == 1.0 && beta == 0.0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
     const bool odd = (a * NB) & 1;
     auto block = [&](auto jc) {
         constexpr int jl = J0 + decltype(jc)::value;
-        if constexpr (jl <= J1 && jl < GJ && jl - J0 < epi_slots<NB>()) {
+        if constexpr (jl <= J1 && jl < GJ) {
             const int32_t blk = cid[jl - J0];
             if (blk < 0) return;
             constexpr int B0 = jl * NB < H0 ? H0 - jl * NB : 0;
-            constexpr int B1 = (jl + 1) * NB > H0 + 32 ? H0 + 32 - jl * NB : NB;
+            constexpr int B1 = (jl + 1) * NB > H0 + W ? H0 + W - jl * NB : NB;
             double *dst = C + (int64_t)blk * c_stride + a * NB;
             double w[NB];
 #pragma unroll
@@ -262,7 +265,7 @@ __device__ __forceinline__ void write_rows(double *C, int c_stride, double alpha
             }
         }
     };
-    static_assert(J1 - J0 < 9, "slots of a half");
+    static_assert(J1 - J0 < 9 && J1 - J0 < epi_slots<NB, W>(), "slots of a thread's columns");
     block(std::integral_constant<int, 0>());
     block(std::integral_constant<int, 1>());
     block(std::integral_constant<int, 2>());
@@ -363,6 +366,41 @@ __device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *
             const uint32_t c = cg - 1 - k;
             if (!bar_wait_plain(smem_u32(&bars->full[c % NS]), (c / NS) & 1u)) *abort_flag = 1;
         }
+    __syncwarp();
+}
+
+// The scheduler warp: hands out the launch's tiles in order, so that the tiles in flight on the
+// GPU stay neighbours (they share the A pieces of one or two M groups) and no CTA idles while
+// others hold several tiles.  nmain(tile): its main K steps.
+template <class Args, class B, class F>
+__device__ __forceinline__ void schedule(const Args &p, B *bars, volatile int *abort_flag, int lane,
+                                         F nmain)
+{
+    if (lane == 0) {
+        int i = blockIdx.x;
+        for (uint32_t n = 0;; ++n) {
+            TileRec r;
+            r.tile = -1;
+            r.s0 = 0;
+            r.nks = r.nm = 0;
+            if (i < p.n_tiles) {
+                r.tile = i;
+                r.s0 = p.kstart[i];
+                r.nks = (int)(p.kstart[i + 1] - r.s0);
+                r.nm = nmain(i);
+            }
+            if (n >= (uint32_t)NTQ &&
+                !bar_wait(smem_u32(&bars->tile_empty[n % NTQ]), ((n / NTQ) + 1) & 1u, abort_flag))
+                break;
+            bars->rec[n % NTQ] = r;
+            bar_arrive(smem_u32(&bars->tile_full[n % NTQ]));
+            if (r.tile < 0) break;
+            i = (int)gridDim.x + (int)atomicAdd(&p.counter[0], 1u);
+        }
+        // the last CTA to finish handing out resets the counters for the next launch
+        __threadfence();
+        if (atomicInc(&p.counter[1], gridDim.x - 1) == gridDim.x - 1) atomicExch(&p.counter[0], 0u);
+    }
     __syncwarp();
 }
 
@@ -499,36 +537,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
         }
         __syncwarp();
     } else if (warp == W_SCHED) {
-        // ------------------------------------------------------------ scheduler
-        // hands out the launch's tiles in order, so that the tiles in flight on the GPU stay
-        // neighbours (they share the A pieces of one or two M groups) and no CTA idles while
-        // others hold several tiles
-        if (lane == 0) {
-            int i = blockIdx.x;
-            for (uint32_t n = 0;; ++n) {
-                TileRec r;
-                r.tile = -1;
-                r.s0 = 0;
-                r.nks = r.nm = 0;
-                if (i < p.n_tiles) {
-                    r.tile = i;
-                    r.s0 = p.kstart[r.tile];
-                    r.nks = (int)(p.kstart[r.tile + 1] - r.s0);
-                    r.nm = p.nmain[r.tile];
-                }
-                if (n >= (uint32_t)NTQ &&
-                    !bar_wait(smem_u32(&bars->tile_empty[n % NTQ]), ((n / NTQ) + 1) & 1u, abort_flag))
-                    break;
-                bars->rec[n % NTQ] = r;
-                bar_arrive(smem_u32(&bars->tile_full[n % NTQ]));
-                if (r.tile < 0) break;
-                i = (int)gridDim.x + (int)atomicAdd(&p.counter[0], 1u);
-            }
-            // the last CTA to finish handing out resets the counters for the next launch
-            __threadfence();
-            if (atomicInc(&p.counter[1], gridDim.x - 1) == gridDim.x - 1) atomicExch(&p.counter[0], 0u);
-        }
-        __syncwarp();
+        schedule(p, bars, abort_flag, lane, [&](int tile) { return p.nmain[tile]; });
     } else {
         // ------------------------------------------------------------ drain and epilogue
         const int quarter = warp & 3, half = warp >> 2;
@@ -542,7 +551,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             const int tile = tr.tile;
             const int np = (tr.nks + KSTEPS * DRAIN - 1) / (KSTEPS * DRAIN);
             // this row's C blocks, loaded now and used after the tile's last period
-            constexpr int NJ = epi_slots<NB>();
+            constexpr int NJ = epi_slots<NB, 32>();
             int32_t cid[NJ];
             if constexpr (NB > 0) {
                 const int si = arow / NB, j0 = (half * 32) / NB;
@@ -584,9 +593,9 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             if constexpr (NB > 0) {
                 auto v = [&](int x) { return f32_to_f64(hi[x]) + f32_to_f64(lo[x]); };
                 if (half == 0)
-                    write_rows<NB, 0>(p.C, p.c_stride, p.alpha, p.beta, cid, arow, v);
+                    write_rows<NB, 0, 32>(p.C, p.c_stride, p.alpha, p.beta, cid, arow, v);
                 else
-                    write_rows<NB, 1>(p.C, p.c_stride, p.alpha, p.beta, cid, arow, v);
+                    write_rows<NB, 32, 32>(p.C, p.c_stride, p.alpha, p.beta, cid, arow, v);
             } else {
                 write_rows_mixed(p, tile, arow, half, hi, lo);
             }
