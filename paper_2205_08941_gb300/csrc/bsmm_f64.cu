@@ -4,10 +4,9 @@
 // a warp share an item and split its task segment (lane q takes tasks q, q+Q, ...), each
 // keeping the item's NB partial sums in registers; the Q partials are then combined by a
 // fixed xor-shuffle tree, so every C row has exactly one writer (no atomics) and the
-// summation order is fixed (deterministic).  Q is picked from the mean segment length so
-// that long segments (k-sums of ~800 blocks) keep all 32 lanes busy and short ones (~13)
-// do not idle lanes.  The B block of a task is read by the NB lanes that own the rows of
-// the same C block, so it is served from L1 after the first touch.
+// summation order is fixed (deterministic).  Q is picked by pick_q.  The B block of a task is
+// read by the NB lanes that own the rows of the same C block, so it is served from L1 after
+// the first touch.
 #include "cq_internal.cuh"
 
 namespace {
@@ -107,13 +106,18 @@ __device__ __forceinline__ void generic_row(unsigned gmask, int q, int64_t c, in
     }
 }
 
-// Mixed orbital counts (1..16 per atom): item -> C block by binary search over the prefix
-// of block row counts; block offsets from the patterns' val_off.  The row's column count
-// selects an instance with exactly that many accumulators (4, 5, 9, 13: the bases of the
-// mixed-species cells), so no FMA slot or shuffle is spent on absent columns.
+// Mixed orbital counts (1..16 per atom): item -> C block by a search over the prefix of block
+// row counts; block offsets from the patterns' val_off.  The row's column count selects an
+// instance with exactly that many accumulators (4, 5, 9, 13: the bases of the mixed-species
+// cells), so no FMA slot or shuffle is spent on absent columns.  Bound by the FP64 pipe, whose
+// time goes by warp: lanes that run different numbers of terms or different instances idle.
+// So the blocks come sorted by width and a segment's tasks by the orbital count of k (S.X of
+// four cells of 5/9/13 orbitals: 56.5 ms unsorted at q = 8, 45.0 with sorted tasks, 33.1 with
+// both at q = 4; U.X 76.7 -> 50.2 ms, 0.97 of the pipe's 1.26 TFLOP/s).
 template <int Q>
 __global__ void __launch_bounds__(256)
 k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ rowitem,
+                   const int32_t *__restrict__ order,
                    const int64_t *__restrict__ seg, const int2 *__restrict__ tasks,
                    const int32_t *__restrict__ nb, const int32_t *__restrict__ c_row,
                    const int32_t *__restrict__ c_col, const int32_t *__restrict__ a_col,
@@ -125,8 +129,23 @@ k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ row
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t item = gt / Q;
     const int q = (int)(gt % Q);
+    // the block of the CTA's first item, then each thread's among the next 256 / Q
+    __shared__ int64_t first;
+    if (threadIdx.x < 32) {
+        const int64_t i0 = (int64_t)blockIdx.x * (blockDim.x / Q);
+        int64_t lo = 0, hi = n_c;  // largest c with rowitem[c] <= i0: 32 probes at a time
+        while (hi - lo > 1) {
+            const int64_t step = (hi - lo + 31) / 32, at = lo + step * (threadIdx.x + 1);
+            const bool le = at < hi && rowitem[at] <= i0;
+            const int n = __popc(__ballot_sync(0xffffffffu, le));
+            hi = min(hi, lo + step * (n + 1));
+            lo += step * n;
+        }
+        if (threadIdx.x == 0) first = lo;
+    }
+    __syncthreads();
     if (item >= n_items) return;  // whole Q groups leave together (blockDim is a multiple of Q)
-    int64_t lo = 0, hi = n_c;     // largest c with rowitem[c] <= item
+    int64_t lo = first, hi = min(n_c, first + blockDim.x / Q + 1);
     while (hi - lo > 1) {
         int64_t mid = (lo + hi) >> 1;
         if (rowitem[mid] <= item)
@@ -134,8 +153,8 @@ k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ row
         else
             hi = mid;
     }
-    const int64_t c = lo;
-    const int r = (int)(item - rowitem[c]);
+    const int64_t c = order[lo];
+    const int r = (int)(item - rowitem[lo]);
     const int ni = nb[c_row[c]], nj = nb[c_col[c]];
     const unsigned gmask =
         Q == 32 ? 0xffffffffu : (((1u << Q) - 1u) << ((threadIdx.x & 31) & ~(Q - 1)));
@@ -152,11 +171,17 @@ k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ row
 #undef CQ_ROW
 }
 
-int pick_q(const TaskList *tl)
+// Lanes per C row.  Neighbouring lanes of a row read different B blocks, so a load of a warp
+// touches about q cache lines: at q = 16 and 32 the L1 serves one line per clock and the kernel
+// runs at 0.6 of the FP64 pipe (T.V on 216 SZP atoms: 4.02 ms at q = 4, 8.19 at 16); at q = 1
+// short segments end at different times (L.S on 512 atoms: 8.58 ms at q = 4, 9.94 at 1).  So four
+// lanes, two on a 4-orbital basis (S.X on 512 sp atoms: 719 us at 2, 782 at 4), and up to eight
+// while the launch is small (less than 100 k threads) and a lane keeps four tasks, or is tiny.
+int pick_q(const TaskList *tl, int nb)
 {
     const double avg = tl->n_c ? (double)tl->n_tasks / (double)tl->n_c : 0.0;
-    int q = 1;
-    while (q < 32 && q * 8 <= avg) q <<= 1;
+    int q = nb == 4 ? 2 : 4;
+    while (q < 8 && tl->n_items * q < 100000 && (avg >= 8.0 * q || tl->n_items * q < 8000)) q <<= 1;
     return q;
 }
 
@@ -203,7 +228,7 @@ static void launch_f64(cq_ctx *ctx, int q, const TaskList *tl, double alpha,
     const int32_t *nb = pC->geo->nb.as<int32_t>();
 #define CQ_GEN(QQ)                                                                            \
     k_bsmm_f64_generic<QQ><<<grid, 256, 0, s>>>(                                              \
-        n_items, tl->n_c, rowitem, tl->seg.as<int64_t>(), tl->tasks.as<int2>(), nb,           \
+        n_items, tl->n_c, rowitem, tl->c_order.as<int32_t>(), tl->seg.as<int64_t>(), tl->tasks.as<int2>(), nb,           \
         pC->row.as<int32_t>(), pC->col.as<int32_t>(), pA->col.as<int32_t>(),                  \
         pA->val_off.as<int64_t>(), pB->val_off.as<int64_t>(), pC->val_off.as<int64_t>(), A, B, \
         C, alpha, beta)
@@ -231,7 +256,7 @@ static cq_status tune_q(cq_ctx *ctx, const TaskList *tl, const cq_pattern *pA, c
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     float best = 1e30f;
-    int best_q = pick_q(tl);
+    int best_q = cq_lane_split(tl);
     for (int q = 1; q <= 32; q <<= 1) {
         launch_f64(ctx, q, tl, 1.0, pA, A, pB, B, 0.0, pC, (double *)tmp);  // warm
         cudaEventRecord(e0, ctx->stream);
@@ -253,7 +278,7 @@ static cq_status tune_q(cq_ctx *ctx, const TaskList *tl, const cq_pattern *pA, c
     return st;
 }
 
-int cq_lane_split(const TaskList *tl) { return tl->q ? tl->q : pick_q(tl); }
+int cq_lane_split(const TaskList *tl) { return tl->q ? tl->q : pick_q(tl, tl->uniform_nb); }
 
 cq_status cq_bsmm_f64(cq_ctx *ctx, const TaskList *tl, double alpha, const cq_pattern *pA,
                       const double *A, const cq_pattern *pB, const double *B, double beta,

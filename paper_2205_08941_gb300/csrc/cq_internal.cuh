@@ -60,8 +60,10 @@ struct TaskList {
     DevBuf seg;     // int64 [n_c + 1]
     DevBuf tasks;   // int2  [n_tasks]: (A block, B block), filled on first FP64 use
     bool filled = false;
-    DevBuf c_rowitem;  // int64 [n_c + 1] prefix of n_i over C blocks (bases other than 4, 9)
+    // bases other than 4, 9: C blocks by width (int32 [n_c]), and the prefix of their rows
+    DevBuf c_order, c_rowitem;  // c_rowitem: int64 [n_c + 1], in the order of c_order
     int64_t n_items = 0;  // scalar C rows (sum of n_i over C blocks)
+    int uniform_nb = 0;   // orbitals per atom of a uniform basis, else 0
     mutable int q = 0;    // lanes per C row of the FP64 kernel chosen by the autotuner (0: none)
 };
 
@@ -165,7 +167,7 @@ cq_status cq_bsmm_f64(cq_ctx *ctx, const TaskList *tl, double alpha, const cq_pa
                       const double *A, const cq_pattern *pB, const double *B, double beta,
                       const cq_pattern *pC, double *C);
 // Lane split the FP64 kernel uses for a task list (tuned if the autotuner ran, else the
-// mean-segment heuristic).
+// rule of pick_q).
 int cq_lane_split(const TaskList *tl);
 cq_status cq_bsmm_split(cq_ctx *ctx, const TaskList *tl, double alpha, const cq_pattern *pA,
                         const double *A, const cq_pattern *pB, const double *B, double beta,
