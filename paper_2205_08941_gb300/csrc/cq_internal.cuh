@@ -166,6 +166,12 @@ cq_status cq_get_map(cq_ctx *ctx, const cq_pattern *pSrc, const cq_pattern *pDst
 cq_status cq_bsmm_f64(cq_ctx *ctx, const TaskList *tl, double alpha, const cq_pattern *pA,
                       const double *A, const cq_pattern *pB, const double *B, double beta,
                       const cq_pattern *pC, double *C);
+// C0 = beta C0 + alpha A0.B0 and C1 = beta C1 + alpha A1.B1 over the same patterns in one launch
+// (a small cell's products leave most of the GPU idle).
+cq_status cq_bsmm_f64_pair(cq_ctx *ctx, const TaskList *tl, double alpha, const cq_pattern *pA,
+                           const double *A0, const double *A1, const cq_pattern *pB,
+                           const double *B0, const double *B1, double beta, const cq_pattern *pC,
+                           double *C0, double *C1);
 // Lane split the FP64 kernel uses for a task list (tuned if the autotuner ran, else the
 // rule of pick_q).
 int cq_lane_split(const TaskList *tl);

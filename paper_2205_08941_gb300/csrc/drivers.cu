@@ -41,6 +41,21 @@ cq_status bsmm(cq_ctx *ctx, double alpha, const cq_pattern *pA, const double *A,
         if (_st != CQ_OK) return _st;      \
     } while (0)
 
+// Two products over the same patterns, C0 = A0.B0 and C1 = A1.B1: one launch in FP64
+cq_status bsmm2(cq_ctx *ctx, const cq_pattern *pA, const double *A0, const double *A1,
+                const cq_pattern *pB, const double *B0, const double *B1, const cq_pattern *pC,
+                double *C0, double *C1, cq_precision prec, double *flops)
+{
+    if (prec != CQ_FP64) {
+        CQ_TRY(bsmm(ctx, 1.0, pA, A0, pB, B0, 0.0, pC, C0, prec, flops));
+        return bsmm(ctx, 1.0, pA, A1, pB, B1, 0.0, pC, C1, prec, flops);
+    }
+    TaskList *tl = nullptr;
+    CQ_TRY(cq_get_tasks(ctx, pA, pB, pC, &tl));
+    *flops += 2.0 * tl->flops;
+    return cq_bsmm_f64_pair(ctx, tl, 1.0, pA, A0, A1, pB, B0, B1, 0.0, pC, C0, C1);
+}
+
 // Quantity q of a per-cell reduction lands in slots [q*nc, q*nc + nc).
 cq_status dot_q(cq_ctx *ctx, const cq_pattern *p, const double *a, const double *b, int q)
 {
@@ -387,11 +402,9 @@ cq_status lnv_energy_number(cq_lnv *s, const double *Lsrc, std::vector<double> &
     double *X = s->X.as<double>(), *Y = s->Y.as<double>(), *U = s->U.as<double>();
     double *R1 = s->R1.as<double>(), *R3 = s->R3.as<double>();
     CQ_TRY(run_phase(s, 1, Lsrc, [&]() -> cq_status {
-        CQ_TRY(bsmm(ctx, 1.0, s->pL, Lsrc, s->pS, s->S, 0.0, s->pX, X, s->prec, &s->flops));
-        CQ_TRY(bsmm(ctx, 1.0, s->pL, Lsrc, s->pS, s->H, 0.0, s->pX, Y, s->prec, &s->flops));
+        CQ_TRY(bsmm2(ctx, s->pL, Lsrc, Lsrc, s->pS, s->S, s->H, s->pX, X, Y, s->prec, &s->flops));
         CQ_TRY(bsmm(ctx, 1.0, s->pS, s->S, s->pX, X, 0.0, s->pU, U, s->prec, &s->flops));
-        CQ_TRY(bsmm(ctx, 1.0, s->pU, U, s->pX, Y, 0.0, s->pL, R1, s->prec, &s->flops));
-        CQ_TRY(bsmm(ctx, 1.0, s->pU, U, s->pX, X, 0.0, s->pL, R3, s->prec, &s->flops));
+        CQ_TRY(bsmm2(ctx, s->pU, U, U, s->pX, Y, X, s->pL, R1, R3, s->prec, &s->flops));
         s->products += 5;
         CQ_TRY(trace_q(ctx, s->pX, X, s->pX, Y, 0));
         CQ_TRY(trace_q(ctx, s->pL, Lsrc, s->pL, R1, 1));
@@ -441,9 +454,8 @@ cq_status lnv_eval_rest(cq_lnv *s)
     double *Z = s->Z.as<double>(), *R1 = s->R1.as<double>(), *R2 = s->R2.as<double>();
     CQ_TRY(run_phase(s, 3, s->L, [&]() -> cq_status {
         CQ_TRY(bsmm(ctx, 1.0, s->pL, s->L, s->pS, s->H, 0.0, s->pX, Y, s->prec, &s->flops));
-        CQ_TRY(bsmm(ctx, 1.0, s->pU, U, s->pX, Y, 0.0, s->pL, R1, s->prec, &s->flops));
         CQ_TRY(bsmm(ctx, 1.0, s->pS, s->S, s->pX, Y, 0.0, s->pU, Z, s->prec, &s->flops));
-        CQ_TRY(bsmm(ctx, 1.0, s->pU, Z, s->pX, X, 0.0, s->pL, R2, s->prec, &s->flops));
+        CQ_TRY(bsmm2(ctx, s->pU, U, Z, s->pX, Y, X, s->pL, R1, R2, s->prec, &s->flops));
         s->products += 4;
         CQ_TRY(trace_q(ctx, s->pX, X, s->pX, Y, 0));
         CQ_TRY(trace_q(ctx, s->pL, s->L, s->pL, R1, 1));
