@@ -101,9 +101,8 @@ struct cq_ctx {
     uint64_t next_id = 1;
     int num_sms = 0;
     DevBuf flag;                     // int32 device error word
-    DevBuf red;                      // reduction partials
-    DevBuf red_out;                  // reduction results (pinned-copy source)
-    double *host_out = nullptr;      // pinned host scalars
+    DevBuf red_count;                // uint32 arrivals of a reduction's CTAs (zero between launches)
+    double *host_out = nullptr;      // pinned host scalars; the last one is the error word
     std::map<std::tuple<uint64_t, uint64_t, uint64_t>, std::unique_ptr<TaskList>> tasks;
     std::map<std::tuple<uint64_t, uint64_t, int>, std::unique_ptr<DevBuf>> maps;
     std::map<std::pair<uint64_t, std::vector<double>>, cq_pattern *> derived;
@@ -183,41 +182,39 @@ cq_status cq_bsmm_emu(cq_ctx *ctx, const TaskList *tl, double alpha, const cq_pa
                       const cq_pattern *pC, double *C);
 
 // ---------------------------------------------------------------- reductions (reduce.cu)
-// All scalar results land in ctx->red_out[slot] on the device; cq_fetch copies them out.
-cq_status cq_trace_dev(cq_ctx *ctx, const cq_pattern *pA, const double *A,
-                       const cq_pattern *pB, const double *B, int slot);
-cq_status cq_dot_dev(cq_ctx *ctx, const cq_pattern *p, const double *A, const double *B,
-                     int slot);
-cq_status cq_frob2_minus_identity_dev(cq_ctx *ctx, const cq_pattern *p, const double *M,
-                                      int slot);
-// slots: [slot] = min(centre - radius), [slot+1] = max(centre + radius), [slot+2] = max |row|
-cq_status cq_row_bounds_dev(cq_ctx *ctx, const cq_pattern *p, const double *M, int slot);
+// A quantity: Tr(A.B), <A, B> (pB unused) or ||A - I||_F^2 (B, pB unused).
+enum RedKind { RED_TRACE = 0, RED_DOT = 1, RED_FROB_MI = 2 };
+struct RedQ {
+    int kind;
+    const cq_pattern *pA;
+    const double *A;
+    const cq_pattern *pB;
+    const double *B;
+};
+constexpr int RED_Q = 4;  // quantities of one launch
+// nq <= RED_Q quantities over one set of atoms in one launch.  The kernel writes the scalars to
+// the pinned slots [slot + e*n + c], c over the n cells of the patterns (per_cell) or n = 1 for
+// the whole; cq_fetch waits for them.
+cq_status cq_reduce(cq_ctx *ctx, int nq, const RedQ *q, bool per_cell, int slot);
+// slots: [slot + 3c] = min(centre - radius), [+1] = max(centre + radius), [+2] = max |row|
+cq_status cq_row_bounds_dev(cq_ctx *ctx, const cq_pattern *p, const double *M, bool per_cell,
+                            int slot);
 cq_status cq_fetch(cq_ctx *ctx, int first, int count, double *host);
 
 // ---------------------------------------------------------------- elementwise (reduce.cu)
-// y <- a*x + b*y over n doubles (b == 0: y not read)
-cq_status cq_axpby(cq_ctx *ctx, int64_t n, double a, const double *x, double b, double *y);
+// y <- a*x + b*z over n doubles (y may be x or z; b == 0: z not read)
+cq_status cq_lincomb(cq_ctx *ctx, int64_t n, double a, const double *x, double b, const double *z,
+                     double *y);
 // dst <- s * (src_ij or src_ji^T) + b * dst on pDst; absent source blocks read as zero
 cq_status cq_gather(cq_ctx *ctx, const cq_pattern *pSrc, const double *src,
                     const cq_pattern *pDst, double *dst, int transpose, double s, double b);
 // M <- s * I on the diagonal blocks of p, zero elsewhere
 cq_status cq_set_identity(cq_ctx *ctx, const cq_pattern *p, double *M, double s);
-// G_E = 2[3(Z + Z^T) - 2(R1 + R1^T + R2)], G_N = 12(U - R3) on P_L
-cq_status cq_lnv_gradients(cq_ctx *ctx, const cq_pattern *pL, const cq_pattern *pU,
-                           const double *Z, const double *U, const double *R1,
-                           const double *R2, const double *R3, double *GE, double *GN);
 
 // ---------------------------------------------------------------- per-cell (batches)
-// One result per cell into red_out[slot + c] (n_cells > 1; contiguous segments).
-cq_status cq_trace_seg_dev(cq_ctx *ctx, const cq_pattern *pA, const double *A,
-                           const cq_pattern *pB, const double *B, int slot);
-cq_status cq_dot_seg_dev(cq_ctx *ctx, const cq_pattern *p, const double *A, const double *B,
-                         int slot);
-// per cell: [slot + 3c] = min(centre - radius), [+1] = max(centre + radius), [+2] = max |row|
-cq_status cq_row_bounds_seg_dev(cq_ctx *ctx, const cq_pattern *p, const double *M, int slot);
-// y <- a[c]*x + b[c]*y on each cell's values (coefficients copied from the host)
-cq_status cq_axpby_seg(cq_ctx *ctx, const cq_pattern *p, const double *a, const double *x,
-                       const double *b, double *y);
+// y <- a[c]*x + b[c]*z on each cell's values (coefficients copied from the host)
+cq_status cq_lincomb_seg(cq_ctx *ctx, const cq_pattern *p, const double *a, const double *x,
+                         const double *b, const double *z, double *y);
 // M <- s[c] * I on each cell's diagonal blocks, zero elsewhere
 cq_status cq_set_identity_seg(cq_ctx *ctx, const cq_pattern *p, double *M, const double *s);
 

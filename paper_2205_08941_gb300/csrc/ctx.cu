@@ -193,12 +193,12 @@ constexpr int32_t CQ_FLAG_WAIT_TIMEOUT = 16;
 cq_status cq_read_flag(cq_ctx *ctx, int32_t *flag)
 {
     cq_status st = cq_check_cuda(
-        ctx, cudaMemcpyAsync(ctx->host_out, ctx->flag.ptr, sizeof(int32_t),
+        ctx, cudaMemcpyAsync(ctx->host_out + CQ_RED_SLOTS - 1, ctx->flag.ptr, sizeof(int32_t),
                              cudaMemcpyDeviceToHost, ctx->stream), "flag read");
     if (st != CQ_OK) return st;
     st = cq_check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "sync");
     if (st != CQ_OK) return st;
-    std::memcpy(flag, ctx->host_out, sizeof(int32_t));
+    std::memcpy(flag, ctx->host_out + CQ_RED_SLOTS - 1, sizeof(int32_t));
     if (!*flag) return CQ_OK;
     st = cq_check_cuda(ctx, cudaMemsetAsync(ctx->flag.ptr, 0, 4, ctx->stream), "flag");
     if (st == CQ_OK && (*flag & CQ_FLAG_WAIT_TIMEOUT))
@@ -226,19 +226,15 @@ static cq_status check_async_flag(cq_ctx *ctx)
                    "split product: a tensor-core wait ran out; the result is incomplete");
 }
 
+// The reduction that computed the scalars wrote them, and the error word as its predecessors on
+// the stream left it, to pinned memory: all that is left is to wait.
 cq_status cq_fetch(cq_ctx *ctx, int first, int count, double *host)
 {
-    cq_status st = cq_check_cuda(
-        ctx, cudaMemcpyAsync(ctx->host_out, ctx->red_out.as<double>() + first,
-                             sizeof(double) * count, cudaMemcpyDeviceToHost, ctx->stream),
-        "scalar read");
-    if (st != CQ_OK) return st;
-    if ((st = queue_flag_read(ctx)) != CQ_OK) return st;
-    st = cq_check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "sync");
+    cq_status st = cq_check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "sync");
     if (st != CQ_OK) return st;
     if ((st = check_async_flag(ctx)) != CQ_OK) return st;
     for (int e = 0; e < count; ++e) {
-        host[e] = ctx->host_out[e];
+        host[e] = ctx->host_out[first + e];
         if (!std::isfinite(host[e]))
             return cq_fail(ctx, CQ_ERR_NUMERIC, "non-finite scalar result");
     }
@@ -262,13 +258,14 @@ extern "C" cq_status cq_ctx_create(int device, void *cuda_stream, cq_ctx **out)
     ctx->stream = (cudaStream_t)cuda_stream;
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (cq_alloc(ctx, ctx->flag, 16) != CQ_OK ||
-        cq_alloc(ctx, ctx->red_out, CQ_RED_SLOTS * 8) != CQ_OK ||
+        cq_alloc(ctx, ctx->red_count, CQ_RED_SLOTS * 4) != CQ_OK ||
         cudaMallocHost(&ctx->host_out, CQ_RED_SLOTS * sizeof(double)) != cudaSuccess) {
         delete ctx;
         return CQ_ERR_NOMEM;
     }
     cudaMemsetAsync(ctx->flag.ptr, 0, 16, ctx->stream);
-    cudaMemsetAsync(ctx->red_out.ptr, 0, CQ_RED_SLOTS * 8, ctx->stream);
+    cudaMemsetAsync(ctx->red_count.ptr, 0, CQ_RED_SLOTS * 4, ctx->stream);
+    ctx->host_out[CQ_RED_SLOTS - 1] = 0.0;
     *out = ctx;
     return CQ_OK;
 }
@@ -592,7 +589,8 @@ extern "C" cq_status cq_trace_prod(cq_ctx *ctx, const cq_pattern *pA, const doub
     if (!ctx || !out_host) return CQ_ERR_INVALID;
     cq_status st = check_triple(ctx, pA, pB, pB);
     if (st != CQ_OK) return st;
-    if ((st = cq_trace_dev(ctx, pA, A, pB, B, 0)) != CQ_OK) return st;
+    const RedQ q = {RED_TRACE, pA, A, pB, B};
+    if ((st = cq_reduce(ctx, 1, &q, false, 0)) != CQ_OK) return st;
     return cq_fetch(ctx, 0, 1, out_host);
 }
 
@@ -601,7 +599,8 @@ extern "C" cq_status cq_dot(cq_ctx *ctx, const cq_pattern *p, const double *A, c
 {
     if (!ctx || !p || !out_host) return CQ_ERR_INVALID;
     if (p->ctx != ctx) return cq_fail(ctx, CQ_ERR_PATTERN, "pattern of another context");
-    cq_status st = cq_dot_dev(ctx, p, A, B, 0);
+    const RedQ q = {RED_DOT, p, A, p, B};
+    cq_status st = cq_reduce(ctx, 1, &q, false, 0);
     if (st != CQ_OK) return st;
     return cq_fetch(ctx, 0, 1, out_host);
 }
@@ -745,9 +744,11 @@ extern "C" cq_status cq_peak_fp64(cq_ctx *ctx, double *flops_per_s_host)
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
-    double *sink = ctx->red_out.as<double>() + 63;
+    void *v;
+    cq_status st = cq_scratch(ctx, "peak_sink", sizeof(double), &v);
+    if (st != CQ_OK) return st;
+    double *sink = (double *)v;
     double best = 0.0;
-    cq_status st = CQ_OK;
     for (int kind = 0; kind < 2 && st == CQ_OK; ++kind) {
         const int it = kind == 0 ? iters : iters / 4;
         auto launch = [&](double seed) {

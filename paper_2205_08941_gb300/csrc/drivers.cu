@@ -9,6 +9,7 @@
 // product covers all cells in one launch.  A single cell uses the unsegmented kernels.
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 
 #include "cq_internal.cuh"
 
@@ -56,19 +57,20 @@ cq_status bsmm2(cq_ctx *ctx, const cq_pattern *pA, const double *A0, const doubl
     return cq_bsmm_f64_pair(ctx, tl, 1.0, pA, A0, A1, pB, B0, B1, 0.0, pC, C0, C1);
 }
 
-// Quantity q of a per-cell reduction lands in slots [q*nc, q*nc + nc).
-cq_status dot_q(cq_ctx *ctx, const cq_pattern *p, const double *a, const double *b, int q)
+RedQ trace_of(const cq_pattern *pA, const double *A, const cq_pattern *pB, const double *B)
 {
-    const int nc = p->n_cells();
-    return nc == 1 ? cq_dot_dev(ctx, p, a, b, q) : cq_dot_seg_dev(ctx, p, a, b, q * nc);
+    return {RED_TRACE, pA, A, pB, B};
 }
 
-cq_status trace_q(cq_ctx *ctx, const cq_pattern *pA, const double *A, const cq_pattern *pB,
-                  const double *B, int q)
+RedQ dot_of(const cq_pattern *p, const double *a, const double *b)
 {
-    const int nc = pA->n_cells();
-    return nc == 1 ? cq_trace_dev(ctx, pA, A, pB, B, q)
-                   : cq_trace_seg_dev(ctx, pA, A, pB, B, q * nc);
+    return {RED_DOT, p, a, p, b};
+}
+
+// Quantities of every cell in one launch; quantity q of cell c lands in slot q*nc + c.
+cq_status reduce_q(cq_ctx *ctx, std::initializer_list<RedQ> q)
+{
+    return cq_reduce(ctx, (int)q.size(), q.begin(), true, 0);
 }
 
 // nq quantities of nc cells: out[q][c]
@@ -82,12 +84,12 @@ cq_status fetch_q(cq_ctx *ctx, int nc, int nq, std::vector<std::vector<double>> 
     return CQ_OK;
 }
 
-// y <- a_c x + b_c y on every cell of p
-cq_status axpby_c(cq_ctx *ctx, const cq_pattern *p, const std::vector<double> &a,
-                  const double *x, const std::vector<double> &b, double *y)
+// y <- a_c x + b_c z on every cell of p
+cq_status lin_c(cq_ctx *ctx, const cq_pattern *p, const std::vector<double> &a, const double *x,
+                const std::vector<double> &b, const double *z, double *y)
 {
-    if (p->n_cells() == 1) return cq_axpby(ctx, p->n_values, a[0], x, b[0], y);
-    return cq_axpby_seg(ctx, p, a.data(), x, b.data(), y);
+    if (p->n_cells() == 1) return cq_lincomb(ctx, p->n_values, a[0], x, b[0], z, y);
+    return cq_lincomb_seg(ctx, p, a.data(), x, b.data(), z, y);
 }
 
 cq_status copy_vals(cq_ctx *ctx, double *dst, const double *src, int64_t n)
@@ -107,13 +109,13 @@ extern "C" cq_status cq_hotelling_init(cq_ctx *ctx, const cq_pattern *pS, const 
     CQ_TRY(same_ctx(ctx, pS, pT));
     const int nc = pS->n_cells();
     if (nc == 1) {
-        CQ_TRY(cq_row_bounds_dev(ctx, pS, S, 0));
+        CQ_TRY(cq_row_bounds_dev(ctx, pS, S, false, 0));
         double b[3];
         CQ_TRY(cq_fetch(ctx, 0, 3, b));
         if (!(b[2] > 0.0)) return cq_fail(ctx, CQ_ERR_NUMERIC, "hotelling_init: S has a zero row");
         return cq_set_identity(ctx, pT, T, 1.0 / b[2]);
     }
-    CQ_TRY(cq_row_bounds_seg_dev(ctx, pS, S, 0));
+    CQ_TRY(cq_row_bounds_dev(ctx, pS, S, true, 0));
     std::vector<double> b(3 * nc), inv(nc);
     CQ_TRY(cq_fetch(ctx, 0, 3 * nc, b.data()));
     for (int c = 0; c < nc; ++c) {
@@ -136,9 +138,10 @@ extern "C" cq_status cq_hotelling_step(cq_ctx *ctx, const cq_pattern *pS, const 
     CQ_TRY(cq_scratch(ctx, "hot_W", sizeof(double) * pT->n_values, &w));
     double *V = (double *)v, *W = (double *)w;
     CQ_TRY(bsmm(ctx, 1.0, pS, S, pT, T, 0.0, pV, V, CQ_FP64));
-    CQ_TRY(cq_frob2_minus_identity_dev(ctx, pV, V, 0));
+    const RedQ fq = {RED_FROB_MI, pV, V, pV, nullptr};
+    CQ_TRY(cq_reduce(ctx, 1, &fq, false, 0));
     CQ_TRY(bsmm(ctx, 1.0, pT, T, pV, V, 0.0, pT, W, CQ_FP64));
-    CQ_TRY(cq_axpby(ctx, pT->n_values, -1.0, W, 2.0, T));
+    CQ_TRY(cq_lincomb(ctx, pT->n_values, -1.0, W, 2.0, T, T));
     double r2;
     CQ_TRY(cq_fetch(ctx, 0, 1, &r2));
     if (resid_host) *resid_host = std::sqrt(r2);
@@ -176,10 +179,9 @@ extern "C" cq_status cq_overlap_inverse_cg(cq_ctx *ctx, const cq_pattern *pS, co
     int32_t k = 0;
     for (;; ++k) {
         CQ_TRY(bsmm(ctx, 1.0, pS, S, pV, R, 0.0, pT, W, CQ_FP64));
-        CQ_TRY(cq_axpby(ctx, nT, -1.0, W, 0.0, G));
+        CQ_TRY(cq_lincomb(ctx, nT, -1.0, W, 0.0, G, G));
         CQ_TRY(cq_gather(ctx, pT, W, pT, G, 1, -1.0, 1.0));      // G = -(W + W^T)
-        CQ_TRY(cq_dot_dev(ctx, pT, G, G, 0));
-        CQ_TRY(cq_dot_dev(ctx, pV, R, R, 1));
+        CQ_TRY(reduce_q(ctx, {dot_of(pT, G, G), dot_of(pV, R, R)}));
         double v[2];
         CQ_TRY(cq_fetch(ctx, 0, 2, v));
         if (!std::isfinite(v[0]) || !std::isfinite(v[1]))
@@ -190,17 +192,16 @@ extern "C" cq_status cq_overlap_inverse_cg(cq_ctx *ctx, const cq_pattern *pS, co
         if (iters_host) *iters_host = k;  // entries 0..k of the histories hold values
         if (k == 0) g0 = gn;
         if (k == max_iter || gn <= gtol * g0) break;
-        CQ_TRY(cq_axpby(ctx, nT, -1.0, G, k == 0 ? 0.0 : v[0] / gg_prev, D));
+        CQ_TRY(cq_lincomb(ctx, nT, -1.0, G, k == 0 ? 0.0 : v[0] / gg_prev, D, D));
         CQ_TRY(bsmm(ctx, 1.0, pS, S, pT, D, 0.0, pV, SD, CQ_FP64));
-        CQ_TRY(cq_dot_dev(ctx, pT, G, D, 0));
-        CQ_TRY(cq_dot_dev(ctx, pV, SD, SD, 1));
+        CQ_TRY(reduce_q(ctx, {dot_of(pT, G, D), dot_of(pV, SD, SD)}));
         double q[2];
         CQ_TRY(cq_fetch(ctx, 0, 2, q));
         if (!(q[1] > 0.0) || !std::isfinite(q[0]))
             return cq_fail(ctx, CQ_ERR_NUMERIC, "overlap_inverse_cg: degenerate direction");
         const double a = -q[0] / (2.0 * q[1]);
-        CQ_TRY(cq_axpby(ctx, nT, a, D, 1.0, T));
-        CQ_TRY(cq_axpby(ctx, nV, -a, SD, 1.0, R));
+        CQ_TRY(cq_lincomb(ctx, nT, a, D, 1.0, T, T));
+        CQ_TRY(cq_lincomb(ctx, nV, -a, SD, 1.0, R, R));
         gg_prev = v[0];
     }
     return CQ_OK;
@@ -230,8 +231,8 @@ extern "C" cq_status cq_pm_guess_cells(cq_ctx *ctx, const cq_pattern *pS, const 
     CQ_TRY(bsmm(ctx, 1.0, pT, T, pS, H, 0.0, pX, TH, CQ_FP64));
     if (nc == 1) {
         const double n_orb = (double)pS->geo->n_orb, n_occ = n_occ_host[0];
-        CQ_TRY(cq_trace_dev(ctx, pT, T, pS, H, 0));
-        CQ_TRY(cq_row_bounds_dev(ctx, pX, TH, 1));
+        CQ_TRY(reduce_q(ctx, {trace_of(pT, T, pS, H)}));
+        CQ_TRY(cq_row_bounds_dev(ctx, pX, TH, false, 1));
         double sc[4];
         CQ_TRY(cq_fetch(ctx, 0, 4, sc));
         const double mu = sc[0] / n_orb;
@@ -240,8 +241,8 @@ extern "C" cq_status cq_pm_guess_cells(cq_ctx *ctx, const cq_pattern *pS, const 
         CQ_TRY(bsmm(ctx, -lam / n_orb, pX, TH, pT, T, 0.0, pL, L, CQ_FP64));
         return cq_gather(ctx, pT, T, pL, L, 0, lam * mu / n_orb + n_occ / n_orb, 1.0);
     }
-    CQ_TRY(cq_trace_seg_dev(ctx, pT, T, pS, H, 0));
-    CQ_TRY(cq_row_bounds_seg_dev(ctx, pX, TH, nc));
+    CQ_TRY(reduce_q(ctx, {trace_of(pT, T, pS, H)}));
+    CQ_TRY(cq_row_bounds_dev(ctx, pX, TH, true, nc));
     std::vector<double> sc(4 * nc);
     CQ_TRY(cq_fetch(ctx, 0, 4 * nc, sc.data()));
     std::vector<double> a(nc), b(nc), one(nc, 1.0), zero(nc, 0.0);
@@ -255,11 +256,11 @@ extern "C" cq_status cq_pm_guess_cells(cq_ctx *ctx, const cq_pattern *pS, const 
     }
     // L = a_c THT + b_c T on P_L
     CQ_TRY(bsmm(ctx, 1.0, pX, TH, pT, T, 0.0, pL, L, CQ_FP64));
-    CQ_TRY(axpby_c(ctx, pL, a, L, zero, L));
+    CQ_TRY(lin_c(ctx, pL, a, L, zero, L, L));
     void *tl;
     CQ_TRY(cq_scratch(ctx, "pm_TL", sizeof(double) * pL->n_values, &tl));
     CQ_TRY(cq_gather(ctx, pT, T, pL, (double *)tl, 0, 1.0, 0.0));
-    return axpby_c(ctx, pL, b, (double *)tl, one, L);
+    return lin_c(ctx, pL, b, (double *)tl, one, L, L);
 }
 
 extern "C" cq_status cq_pm_guess(cq_ctx *ctx, const cq_pattern *pS, const double *S,
@@ -406,10 +407,8 @@ cq_status lnv_energy_number(cq_lnv *s, const double *Lsrc, std::vector<double> &
         CQ_TRY(bsmm(ctx, 1.0, s->pS, s->S, s->pX, X, 0.0, s->pU, U, s->prec, &s->flops));
         CQ_TRY(bsmm2(ctx, s->pU, U, U, s->pX, Y, X, s->pL, R1, R3, s->prec, &s->flops));
         s->products += 5;
-        CQ_TRY(trace_q(ctx, s->pX, X, s->pX, Y, 0));
-        CQ_TRY(trace_q(ctx, s->pL, Lsrc, s->pL, R1, 1));
-        CQ_TRY(trace_q(ctx, s->pX, X, s->pX, X, 2));
-        return trace_q(ctx, s->pL, Lsrc, s->pL, R3, 3);
+        return reduce_q(ctx, {trace_of(s->pX, X, s->pX, Y), trace_of(s->pL, Lsrc, s->pL, R1),
+                              trace_of(s->pX, X, s->pX, X), trace_of(s->pL, Lsrc, s->pL, R3)});
     }));
     std::vector<std::vector<double>> t;
     CQ_TRY(fetch_q(ctx, s->nc, 4, t));
@@ -422,10 +421,11 @@ cq_status lnv_energy_number(cq_lnv *s, const double *Lsrc, std::vector<double> &
     return CQ_OK;
 }
 
-// Electron-number half of an evaluation at s->L: X = LS, U = SX, R3 = UX, N and G_N.
+// Electron-number half of an evaluation at s->L: X = LS, U = SX, R3 = UX, N, G_N and
+// gn2 = <G_N, G_N> per cell.
 // (The products and values are those of a full evaluation; E and G_E follow in
 // lnv_eval_rest at the same L.)
-cq_status lnv_eval_n(cq_lnv *s)
+cq_status lnv_eval_n(cq_lnv *s, std::vector<double> &gn2)
 {
     cq_ctx *ctx = s->ctx;
     double *X = s->X.as<double>(), *U = s->U.as<double>(), *R3 = s->R3.as<double>();
@@ -434,20 +434,22 @@ cq_status lnv_eval_n(cq_lnv *s)
         CQ_TRY(bsmm(ctx, 1.0, s->pS, s->S, s->pX, X, 0.0, s->pU, U, s->prec, &s->flops));
         CQ_TRY(bsmm(ctx, 1.0, s->pU, U, s->pX, X, 0.0, s->pL, R3, s->prec, &s->flops));
         s->products += 3;
-        CQ_TRY(trace_q(ctx, s->pX, X, s->pX, X, 0));
-        CQ_TRY(trace_q(ctx, s->pL, s->L, s->pL, R3, 1));
-        return cq_lnv_gradient_n(ctx, s->pL, s->pU, U, R3, s->GN.as<double>());
+        double *GN = s->GN.as<double>();
+        CQ_TRY(cq_lnv_gradient_n(ctx, s->pL, s->pU, U, R3, GN));
+        return reduce_q(ctx, {trace_of(s->pX, X, s->pX, X), trace_of(s->pL, s->L, s->pL, R3),
+                              dot_of(s->pL, GN, GN)});
     }));
     std::vector<std::vector<double>> t;
-    CQ_TRY(fetch_q(ctx, s->nc, 2, t));
+    CQ_TRY(fetch_q(ctx, s->nc, 3, t));
+    gn2 = t[2];
     s->N.resize(s->nc);
     for (int c = 0; c < s->nc; ++c) s->N[c] = 2.0 * (3.0 * t[0][c] - 2.0 * t[1][c]);
     return CQ_OK;
 }
 
 // Energy half at the L of the last lnv_eval_n (X, U still current): Y = LH, R1 = UY,
-// Z = SY, R2 = ZX, E and G_E.
-cq_status lnv_eval_rest(cq_lnv *s)
+// Z = SY, R2 = ZX, E, G_E and gegn = <G_E, G_N> per cell.
+cq_status lnv_eval_rest(cq_lnv *s, std::vector<double> &gegn)
 {
     cq_ctx *ctx = s->ctx;
     double *X = s->X.as<double>(), *Y = s->Y.as<double>(), *U = s->U.as<double>();
@@ -457,12 +459,14 @@ cq_status lnv_eval_rest(cq_lnv *s)
         CQ_TRY(bsmm(ctx, 1.0, s->pS, s->S, s->pX, Y, 0.0, s->pU, Z, s->prec, &s->flops));
         CQ_TRY(bsmm2(ctx, s->pU, U, Z, s->pX, Y, X, s->pL, R1, R2, s->prec, &s->flops));
         s->products += 4;
-        CQ_TRY(trace_q(ctx, s->pX, X, s->pX, Y, 0));
-        CQ_TRY(trace_q(ctx, s->pL, s->L, s->pL, R1, 1));
-        return cq_lnv_gradient_e(ctx, s->pL, s->pU, Z, R1, R2, s->GE.as<double>());
+        double *GE = s->GE.as<double>();
+        CQ_TRY(cq_lnv_gradient_e(ctx, s->pL, s->pU, Z, R1, R2, GE));
+        return reduce_q(ctx, {trace_of(s->pX, X, s->pX, Y), trace_of(s->pL, s->L, s->pL, R1),
+                              dot_of(s->pL, GE, s->GN.as<double>())});
     }));
     std::vector<std::vector<double>> t;
-    CQ_TRY(fetch_q(ctx, s->nc, 2, t));
+    CQ_TRY(fetch_q(ctx, s->nc, 3, t));
+    gegn = t[2];
     s->E.resize(s->nc);
     for (int c = 0; c < s->nc; ++c) s->E[c] = 2.0 * (3.0 * t[0][c] - 2.0 * t[1][c]);
     return CQ_OK;
@@ -471,7 +475,7 @@ cq_status lnv_eval_rest(cq_lnv *s)
 // <a, b> per cell
 cq_status dots(cq_lnv *s, const double *a, const double *b, std::vector<double> &out)
 {
-    CQ_TRY(dot_q(s->ctx, s->pL, a, b, 0));
+    CQ_TRY(reduce_q(s->ctx, {dot_of(s->pL, a, b)}));
     std::vector<std::vector<double>> t;
     CQ_TRY(fetch_q(s->ctx, s->nc, 1, t));
     out = t[0];
@@ -484,9 +488,11 @@ cq_status dots(cq_lnv *s, const double *a, const double *b, std::vector<double> 
 // iterates and decisions are those of "full evaluation, then correct and re-evaluate";
 // only the E half of the intermediate evaluations (never used) is skipped.  In a batch a
 // cell within tolerance receives a zero correction.
-cq_status lnv_evaluate_corrected(cq_lnv *s, std::vector<int> &count)
+// gegn and gn2 are <G_E, G_N> and <G_N, G_N> at that L.
+cq_status lnv_evaluate_corrected(cq_lnv *s, std::vector<int> &count, std::vector<double> &gegn,
+                                 std::vector<double> &gn2)
 {
-    CQ_TRY(lnv_eval_n(s));
+    CQ_TRY(lnv_eval_n(s, gn2));
     count.assign(s->nc, 0);
     // split-BF16 products resolve N to ~1e-10 relative, so their corrections stop at 1e-9
     const double tol = s->prec == CQ_SPLIT_BF16X3 ? s->n_tol_split : s->n_tol;
@@ -498,37 +504,41 @@ cq_status lnv_evaluate_corrected(cq_lnv *s, std::vector<int> &count)
             any = any || need[c];
         }
         if (!any) break;
-        std::vector<double> gn2;
-        CQ_TRY(dots(s, s->GN.as<double>(), s->GN.as<double>(), gn2));
         std::vector<double> a(s->nc, 0.0), one(s->nc, 1.0);
         for (int c = 0; c < s->nc; ++c)
             if (need[c]) {
                 a[c] = (s->ne[c] - s->N[c]) / gn2[c];
                 count[c] += 1;
             }
-        CQ_TRY(axpby_c(s->ctx, s->pL, a, s->GN.as<double>(), one, s->L));
-        CQ_TRY(lnv_eval_n(s));
+        CQ_TRY(lin_c(s->ctx, s->pL, a, s->GN.as<double>(), one, s->L, s->L));
+        CQ_TRY(lnv_eval_n(s, gn2));
     }
-    return lnv_eval_rest(s);
+    return lnv_eval_rest(s, gegn);
 }
 
-// mu_c = <G_E,G_N>/<G_N,G_N> and G = G_E - mu_c G_N into s->G; returns <G_N,G_N> per cell.
-cq_status lnv_mu_g(cq_lnv *s, std::vector<double> &mu, std::vector<double> &gn2)
+// <G_E,G_N> and <G_N,G_N> per cell
+cq_status lnv_gradient_dots(cq_lnv *s, std::vector<double> &gegn, std::vector<double> &gn2)
 {
-    cq_ctx *ctx = s->ctx;
-    CQ_TRY(dot_q(ctx, s->pL, s->GE.as<double>(), s->GN.as<double>(), 0));
-    CQ_TRY(dot_q(ctx, s->pL, s->GN.as<double>(), s->GN.as<double>(), 1));
+    const double *GE = s->GE.as<double>(), *GN = s->GN.as<double>();
+    CQ_TRY(reduce_q(s->ctx, {dot_of(s->pL, GE, GN), dot_of(s->pL, GN, GN)}));
     std::vector<std::vector<double>> d;
-    CQ_TRY(fetch_q(ctx, s->nc, 2, d));
-    mu.resize(s->nc);
+    CQ_TRY(fetch_q(s->ctx, s->nc, 2, d));
+    gegn = d[0];
     gn2 = d[1];
+    return CQ_OK;
+}
+
+// mu_c = <G_E,G_N>/<G_N,G_N> and G = G_E - mu_c G_N into `G`
+cq_status lnv_mu_g(cq_lnv *s, const std::vector<double> &gegn, const std::vector<double> &gn2,
+                   std::vector<double> &mu, double *G)
+{
+    mu.resize(s->nc);
     std::vector<double> neg(s->nc), one(s->nc, 1.0);
     for (int c = 0; c < s->nc; ++c) {
-        mu[c] = d[0][c] / d[1][c];
+        mu[c] = gegn[c] / gn2[c];
         neg[c] = -mu[c];
     }
-    CQ_TRY(copy_vals(ctx, s->G.as<double>(), s->GE.as<double>(), s->pL->n_values));
-    return axpby_c(ctx, s->pL, neg, s->GN.as<double>(), one, s->G.as<double>());
+    return lin_c(s->ctx, s->pL, neg, s->GN.as<double>(), one, s->GE.as<double>(), G);
 }
 
 void cubic_coeffs(double f0, double g, double a1, double f1, double a2, double f2, double *c2,
@@ -551,11 +561,13 @@ bool cubic_min(double w1, double w2, double w3, double *a)
     return *a > 0.0;
 }
 
-cq_status lnv_report(cq_lnv *s, cq_lnv_report *rep)
+// Energy, electron count, mu and gradient norm of the current point, with G in `G`
+cq_status lnv_report(cq_lnv *s, const std::vector<double> &gegn, const std::vector<double> &gn2,
+                     double *G, cq_lnv_report *rep)
 {
-    std::vector<double> mu, gn2, gg;
-    CQ_TRY(lnv_mu_g(s, mu, gn2));
-    CQ_TRY(dots(s, s->G.as<double>(), s->G.as<double>(), gg));
+    std::vector<double> mu, gg;
+    CQ_TRY(lnv_mu_g(s, gegn, gn2, mu, G));
+    CQ_TRY(dots(s, G, G, gg));
     for (int c = 0; c < s->nc; ++c) {
         rep[c].energy = s->E[c];
         rep[c].n_elec = s->N[c];
@@ -602,7 +614,8 @@ extern "C" cq_status cq_lnv_create_cells(cq_ctx *ctx, const cq_pattern *pS, cons
     CQ_TRY(cq_alloc(ctx, s->Z, bu));
     for (DevBuf *b : {&s->R1, &s->R2, &s->R3, &s->GE, &s->GN, &s->G, &s->Gp, &s->D, &s->Dp, &s->Lt})
         CQ_TRY(cq_alloc(ctx, *b, bl));
-    CQ_TRY(lnv_evaluate_corrected(s.get(), s->n_corr_initial));
+    std::vector<double> gegn, gn2;
+    CQ_TRY(lnv_evaluate_corrected(s.get(), s->n_corr_initial, gegn, gn2));
     ctx->live_lnv.push_back(s.get());
     *out = s.release();
     return CQ_OK;
@@ -630,8 +643,9 @@ extern "C" cq_status cq_lnv_step(cq_lnv *s, cq_lnv_report *rep)
     const std::vector<double> one(nc, 1.0), zero(nc, 0.0), neg1(nc, -1.0);
     s->flops = 0.0;
     s->products = 0;
-    std::vector<double> mu, gn2;
-    CQ_TRY(lnv_mu_g(s, mu, gn2));
+    std::vector<double> mu, gegn, gn2;
+    CQ_TRY(lnv_gradient_dots(s, gegn, gn2));
+    CQ_TRY(lnv_mu_g(s, gegn, gn2, mu, G));
     // direction source Zc: G itself, or with a preconditioner Zs = sym(mask_L(T G T)); Zq is
     // the previous step's (G_prev, or Z_prev)
     const double *Zc = G, *Zq = s->Gp.as<double>();
@@ -648,28 +662,31 @@ extern "C" cq_status cq_lnv_step(cq_lnv *s, cq_lnv_report *rep)
     }
     std::vector<bool> restart(nc, !s->have_prev);
     if (!s->have_prev) {
-        CQ_TRY(axpby_c(ctx, pL, neg1, Zc, zero, D));
+        CQ_TRY(lin_c(ctx, pL, neg1, Zc, zero, D, D));
     } else {
         // beta = max(0, <G, Z - Z_prev> / <G_prev, Z_prev>) (Z = G without a preconditioner),
         // D = -Z + beta D_prev
-        CQ_TRY(copy_vals(ctx, D, Zc, n));
-        CQ_TRY(axpby_c(ctx, pL, neg1, Zq, one, D));
-        CQ_TRY(dot_q(ctx, pL, G, D, 0));
-        CQ_TRY(dot_q(ctx, pL, s->Gp.as<double>(), Zq, 1));
+        CQ_TRY(lin_c(ctx, pL, neg1, Zq, one, Zc, D));
+        CQ_TRY(reduce_q(ctx, {dot_of(pL, G, D), dot_of(pL, s->Gp.as<double>(), Zq)}));
         std::vector<std::vector<double>> d;
         CQ_TRY(fetch_q(ctx, nc, 2, d));
         std::vector<double> beta(nc);
         for (int c = 0; c < nc; ++c) beta[c] = std::fmax(0.0, d[0][c] / d[1][c]);
-        CQ_TRY(copy_vals(ctx, D, s->Dp.as<double>(), n));
-        CQ_TRY(axpby_c(ctx, pL, neg1, Zc, beta, D));
+        CQ_TRY(lin_c(ctx, pL, neg1, Zc, beta, s->Dp.as<double>(), D));
     }
     std::vector<double> dg;
     CQ_TRY(dots(s, D, GN, dg));
     std::vector<double> proj(nc);
     for (int c = 0; c < nc; ++c) proj[c] = -(dg[c] / gn2[c]);
-    CQ_TRY(axpby_c(ctx, pL, proj, GN, one, D));
-    std::vector<double> gd;
-    CQ_TRY(dots(s, G, D, gd));
+    CQ_TRY(lin_c(ctx, pL, proj, GN, one, D, D));
+    // <G,D> decides on a restart; <G_E,D> and <G_N,D> hold unless one happens
+    auto slopes = [&](std::vector<std::vector<double>> &t) -> cq_status {
+        CQ_TRY(reduce_q(ctx, {dot_of(pL, GE, D), dot_of(pL, GN, D), dot_of(pL, G, D)}));
+        return fetch_q(ctx, nc, 3, t);
+    };
+    std::vector<std::vector<double>> g2;
+    CQ_TRY(slopes(g2));
+    const std::vector<double> gd = g2[2];
     bool any_restart = false;
     std::vector<double> ra(nc, 0.0), rb(nc, 1.0);
     for (int c = 0; c < nc; ++c)
@@ -679,7 +696,10 @@ extern "C" cq_status cq_lnv_step(cq_lnv *s, cq_lnv_report *rep)
             ra[c] = -1.0;
             rb[c] = 0.0;
         }
-    if (any_restart) CQ_TRY(axpby_c(ctx, pL, ra, Zc, rb, D));
+    if (any_restart) {
+        CQ_TRY(lin_c(ctx, pL, ra, Zc, rb, D, D));
+        CQ_TRY(slopes(g2));
+    }
     std::vector<double> a1(nc), a2(nc);
     if (!s->have_alpha) {
         std::vector<double> gg;
@@ -691,18 +711,12 @@ extern "C" cq_status cq_lnv_step(cq_lnv *s, cq_lnv_report *rep)
     }
     for (int c = 0; c < nc; ++c) a2[c] = 2.0 * a1[c];
     const std::vector<double> E0 = s->E, N0 = s->N;
-    CQ_TRY(dot_q(ctx, pL, GE, D, 0));
-    CQ_TRY(dot_q(ctx, pL, GN, D, 1));
-    std::vector<std::vector<double>> g2;
-    CQ_TRY(fetch_q(ctx, nc, 2, g2));
     const std::vector<double> &gE = g2[0], &gNd = g2[1];
     std::vector<double> E1, N1, E2, N2;
     double *Lt = s->Lt.as<double>();
-    CQ_TRY(copy_vals(ctx, Lt, s->L, n));
-    CQ_TRY(axpby_c(ctx, pL, a1, D, one, Lt));
+    CQ_TRY(lin_c(ctx, pL, a1, D, one, s->L, Lt));
     CQ_TRY(lnv_energy_number(s, Lt, E1, N1));
-    CQ_TRY(copy_vals(ctx, Lt, s->L, n));
-    CQ_TRY(axpby_c(ctx, pL, a2, D, one, Lt));
+    CQ_TRY(lin_c(ctx, pL, a2, D, one, s->L, Lt));
     CQ_TRY(lnv_energy_number(s, Lt, E2, N2));
     std::vector<double> alpha(nc);
     std::vector<bool> ok(nc);
@@ -725,9 +739,9 @@ extern "C" cq_status cq_lnv_step(cq_lnv *s, cq_lnv_report *rep)
                 alpha[c] = std::fmin(alpha[c],
                                      0.01 * std::sqrt((double)pL->seg_scalars[c] / dd[c]));
     }
-    CQ_TRY(axpby_c(ctx, pL, alpha, D, one, s->L));
+    CQ_TRY(lin_c(ctx, pL, alpha, D, one, s->L, s->L));
     std::vector<int> ncorr;
-    CQ_TRY(lnv_evaluate_corrected(s, ncorr));
+    CQ_TRY(lnv_evaluate_corrected(s, ncorr, gegn, gn2));
     std::swap(s->G.ptr, s->Gp.ptr);  // G_prev <- G
     std::swap(s->D.ptr, s->Dp.ptr);  // D_prev <- D
     if (s->precond) std::swap(s->Zs.ptr, s->Zp.ptr);  // Z_prev <- Z
@@ -735,7 +749,7 @@ extern "C" cq_status cq_lnv_step(cq_lnv *s, cq_lnv_report *rep)
     s->have_alpha = true;
     s->alpha_prev = alpha;
     if (rep) {
-        CQ_TRY(lnv_report(s, rep));
+        CQ_TRY(lnv_report(s, gegn, gn2, s->G.as<double>(), rep));
         for (int c = 0; c < nc; ++c) {
             rep[c].alpha = alpha[c];
             rep[c].restart = restart[c] ? 1 : 0;
@@ -756,7 +770,8 @@ extern "C" cq_status cq_lnv_set_precision(cq_lnv *s, cq_precision prec)
     s->prec = prec;
     s->have_prev = false;
     s->have_alpha = false;
-    return lnv_evaluate_corrected(s, s->n_corr_initial);
+    std::vector<double> gegn, gn2;
+    return lnv_evaluate_corrected(s, s->n_corr_initial, gegn, gn2);
 }
 
 extern "C" cq_status cq_lnv_set_preconditioner(cq_lnv *s, const cq_pattern *pT, const double *T)
@@ -786,28 +801,13 @@ extern "C" cq_status cq_lnv_state(const cq_lnv *cs, cq_lnv_report *rep)
     if (!cs || !rep || !cs->ctx) return CQ_ERR_INVALID;
     // the report needs G scratch: use Lt (not part of the state between steps)
     cq_lnv *s = const_cast<cq_lnv *>(cs);
-    cq_ctx *ctx = s->ctx;
-    const int nc = s->nc;
-    CQ_TRY(dot_q(ctx, s->pL, s->GE.as<double>(), s->GN.as<double>(), 0));
-    CQ_TRY(dot_q(ctx, s->pL, s->GN.as<double>(), s->GN.as<double>(), 1));
-    std::vector<std::vector<double>> d;
-    CQ_TRY(fetch_q(ctx, nc, 2, d));
-    std::vector<double> neg(nc), one(nc, 1.0);
-    for (int c = 0; c < nc; ++c) neg[c] = -(d[0][c] / d[1][c]);
-    double *T = s->Lt.as<double>();
-    CQ_TRY(copy_vals(ctx, T, s->GE.as<double>(), s->pL->n_values));
-    CQ_TRY(axpby_c(ctx, s->pL, neg, s->GN.as<double>(), one, T));
-    std::vector<double> gg;
-    CQ_TRY(dots(s, T, T, gg));
-    for (int c = 0; c < nc; ++c) {
+    for (int c = 0; c < s->nc; ++c) {
         rep[c] = cq_lnv_report();
-        rep[c].energy = s->E[c];
-        rep[c].n_elec = s->N[c];
-        rep[c].mu = -neg[c];
-        rep[c].gnorm = std::sqrt(gg[c] / (double)s->pL->seg_scalars[c]);
         rep[c].n_corr = s->n_corr_initial[c];
     }
-    return CQ_OK;
+    std::vector<double> gegn, gn2;
+    CQ_TRY(lnv_gradient_dots(s, gegn, gn2));
+    return lnv_report(s, gegn, gn2, s->Lt.as<double>(), rep);
 }
 
 extern "C" cq_status cq_lnv_step_flops(cq_lnv *s, double *flops_host)

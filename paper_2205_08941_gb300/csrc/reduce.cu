@@ -1,19 +1,29 @@
-// Traces, inner products, norms, Gershgorin bounds (deterministic FP64 two-level
-// reductions) and the elementwise kernels on pattern values.
+// Traces, inner products, norms, Gershgorin bounds (deterministic FP64 reductions) and the
+// elementwise kernels on pattern values.
 //
-// Reductions: stage 1 runs a fixed grid of RED_G CTAs; every thread accumulates its
-// grid-stride share in a fixed order, each CTA combines its threads by a fixed tree into one
-// partial; stage 2 (one CTA) combines the RED_G partials by a fixed tree.  The result does
-// not depend on scheduling, so repeated runs are bitwise identical.  Padding values at the
-// end of odd-sized blocks are never read.
+// A reduction is one launch for up to RED_Q quantities of one basis: every thread accumulates
+// its share in a fixed order, each CTA combines its threads by a fixed tree into one partial,
+// and the last CTA of a quantity (and cell) to arrive folds the partials, again by a fixed
+// tree, and writes the scalar straight to pinned host memory together with the device error
+// word.  Grid and order depend on sizes alone, so repeated runs are bitwise identical.
+// Padding values at the end of odd-sized blocks are never read.
+//
+// Small cells: a two-kernel reduction followed by two 8-byte copies cost 10 us of launches for
+// a few us of work.  With all the sums of an evaluation in one launch and no copies, the
+// reductions of an LNV run of 4 steps at 64 atoms take 53 launches and 0.46 ms (280 launches and
+// 1.4 ms before), and the run 4.5 ms (6.3).
+#include <algorithm>
 #include <cfloat>
 
 #include "cq_internal.cuh"
 
 namespace {
 
-constexpr int RED_G = 1024;
 constexpr int RED_T = 256;
+// CTAs of a quantity: 3 per SM (what 80 registers a thread allow) for one cell, and at least 48
+// for each cell of a batch
+constexpr int RED_G = 456;
+constexpr int RED_CELL = 48;
 
 enum Op { SUM = 0, MIN = 1, MAX = 2 };
 
@@ -50,100 +60,251 @@ __device__ double cta_reduce(double v)
     return v;
 }
 
-// Stage 2: one CTA of RED_T threads folds `n` partials (strided by `stride`) into out.
+// Where the partials meet and the scalars go (see red_sink).
+struct RedSink {
+    double *part;         // per quantity and cell: gridDim.x partials (of NV values)
+    uint32_t *count;      // arrivals per quantity and cell, zero between launches
+    double *out;          // pinned host scalars, from the first slot on
+    const int32_t *flag;  // device error word and its pinned copy
+    int32_t *flag_out;
+};
+
+// True in every thread of the last CTA of (blockIdx.z, blockIdx.y) to get here, after thread 0
+// of each has written its partials.
+__device__ bool last_arrival(const RedSink &k, int64_t unit)
+{
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&k.count[unit], 1u) == gridDim.x - 1;
+        if (last) k.count[unit] = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+__device__ __forceinline__ void publish_flag(const RedSink &k)
+{
+    *k.flag_out = *k.flag;
+}
+
 template <int OP>
-__global__ void k_final(const double *part, int n, int stride, double *out)
+__device__ double fold(const double *part, int stride)
 {
     double v = identity_of<OP>();
-    for (int e = threadIdx.x; e < n; e += RED_T) v = combine<OP>(v, part[(int64_t)e * stride]);
-    v = cta_reduce<OP>(v);
-    if (threadIdx.x == 0) *out = v;
+    for (int e = threadIdx.x; e < (int)gridDim.x; e += RED_T)
+        v = combine<OP>(v, __ldcg(part + (int64_t)e * stride));
+    return cta_reduce<OP>(v);
 }
 
-// Tr(A.B): warp per A block (i, j); B block (j, i) index from bmap (-1: absent).
-__global__ void __launch_bounds__(RED_T)
-k_trace(int64_t nblk, const int32_t *row, const int32_t *col, const int32_t *nb,
-        const int64_t *a_off, const int64_t *b_off, const int64_t *bmap, const double *A,
-        const double *B, double *part)
+struct RedItem {
+    int kind;  // RedKind
+    int64_t nblk;
+    const int64_t *seg;  // block ranges of the cells (null: one range)
+    const int64_t *a_off, *b_off, *bmap;
+    const int32_t *row, *col;
+    const double *A, *B;
+};
+
+struct RedArgs {
+    RedItem it[RED_Q];
+    const int32_t *nb;
+    RedSink sink;
+};
+
+// One CTA's share of a quantity on a uniform basis of NB orbitals.  Offsets need no index loads
+// (the blocks of a uniform basis lie at a fixed stride) and a lane's elements, transposed ones
+// included, have the same place in every block, so four blocks are in flight at once (24 loads
+// per lane for 9 orbitals); the map of the next four arrives meanwhile.  Bound by HBM:
+// a trace and a dot over 4.5 GB each at 4096 atoms take 0.67 ms, 6.7 TB/s (1.02 and 0.89 ms with
+// a warp walking one block at a time through its index arrays).
+template <int KIND, int NB>
+__device__ double sum_uniform(const RedItem &it, int64_t b0, int64_t b1)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5);
-    double s = 0.0;
-    for (int64_t b = w0; b < nblk; b += (int64_t)RED_G * (RED_T / 32)) {
-        const int64_t t = bmap[b];
-        if (t < 0) continue;
-        const int ni = nb[row[b]], nj = nb[col[b]];
-        const double *a = A + a_off[b];
-        const double *bb = B + b_off[t];
-        for (int e = lane; e < ni * nj; e += 32) {
-            const int r = e / nj, q = e - r * nj;
-            s = fma(a[e], bb[q * ni + r], s);
-        }
+    constexpr int E = NB * NB, ST = (E + 1) & ~1, LPB = E >= 32 ? 32 : 16, U = 4;
+    constexpr int EPL = (E + LPB - 1) / LPB;
+    const int sub = threadIdx.x % LPB;
+    int te[EPL];
+#pragma unroll
+    for (int k = 0; k < EPL; ++k) {
+        const int e = sub + k * LPB;
+        te[k] = KIND == RED_TRACE ? (e % NB) * NB + e / NB : e;
     }
-    s = cta_reduce<SUM>(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// <A, B> over the blocks of one pattern (padding skipped).
-__global__ void __launch_bounds__(RED_T)
-k_dot(int64_t nblk, const int32_t *row, const int32_t *col, const int32_t *nb,
-      const int64_t *off, const double *A, const double *B, double *part)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5);
+    const int64_t W = (int64_t)gridDim.x * (RED_T / LPB);
+    const double *__restrict__ A = it.A;
+    const double *__restrict__ B = it.B;
     double s = 0.0;
-    for (int64_t b = w0; b < nblk; b += (int64_t)RED_G * (RED_T / 32)) {
-        const int sz = nb[row[b]] * nb[col[b]];
-        const int64_t o = off[b];
-        for (int e = lane; e < sz; e += 32) s = fma(A[o + e], B[o + e], s);
-    }
-    s = cta_reduce<SUM>(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(RED_T)
-k_frob2_mi(int64_t nblk, const int32_t *row, const int32_t *col, const int32_t *nb,
-           const int64_t *off, const double *M, double *part)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5);
-    double s = 0.0;
-    for (int64_t b = w0; b < nblk; b += (int64_t)RED_G * (RED_T / 32)) {
-        const int i = row[b], j = col[b];
-        const int ni = nb[i], nj = nb[j];
-        const int64_t o = off[b];
-        for (int e = lane; e < ni * nj; e += 32) {
-            double v = M[o + e];
-            if (i == j && (e / nj) == (e % nj)) v -= 1.0;
-            s = fma(v, v, s);
-        }
-    }
-    s = cta_reduce<SUM>(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// Gershgorin data per scalar row: warp per atom row, lane r < n_i owns scalar row r.
-__global__ void __launch_bounds__(RED_T)
-k_row_bounds(int n_atoms, const int64_t *rp, const int32_t *col, const int32_t *nb,
-             const int64_t *off, const double *M, double *part)
-{
-    const int lane = threadIdx.x & 31;
-    const int w0 = blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5);
-    double lo = DBL_MAX, hi = -DBL_MAX, amax = 0.0;
-    for (int i = w0; i < n_atoms; i += RED_G * (RED_T / 32)) {
-        const int ni = nb[i];
-        if (lane >= ni) continue;
-        double centre = 0.0, rad = 0.0, tot = 0.0;
-        for (int64_t b = rp[i]; b < rp[i + 1]; ++b) {
-            const int j = col[b], nj = nb[j];
-            const double *m = M + off[b] + (int64_t)lane * nj;
-            for (int q = 0; q < nj; ++q) {
-                const double v = m[q];
-                tot += fabs(v);
-                if (j == i && q == lane)
-                    centre = v;
+    int64_t b = b0 + (int64_t)blockIdx.x * (RED_T / LPB) + threadIdx.x / LPB;
+    int64_t t[U];
+    auto partner = [&](int64_t x) -> int64_t {
+        if (x >= b1) return -1;
+        if (KIND == RED_TRACE) return __ldg(it.bmap + x);
+        if (KIND == RED_FROB_MI) return it.row[x] == it.col[x];
+        return x;
+    };
+#pragma unroll
+    for (int u = 0; u < U; ++u) t[u] = partner(b + u * W);
+    while (b < b1) {
+        double av[U][EPL], bv[U][EPL];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < EPL; ++k) {
+                const bool ok = t[u] >= 0 && sub + k * LPB < E;
+                av[u][k] = ok ? __ldg(A + (b + u * W) * ST + sub + k * LPB) : 0.0;
+                if (KIND == RED_FROB_MI)
+                    bv[u][k] = ok && t[u] && (sub + k * LPB) % (NB + 1) == 0 ? 1.0 : 0.0;
                 else
-                    rad += fabs(v);
+                    bv[u][k] = ok ? __ldg(B + t[u] * ST + te[k]) : 0.0;
+            }
+        b += U * W;
+#pragma unroll
+        for (int u = 0; u < U; ++u) t[u] = partner(b + u * W);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < EPL; ++k) {
+                if (KIND == RED_FROB_MI) {
+                    const double v = av[u][k] - bv[u][k];
+                    s = fma(v, v, s);
+                } else {
+                    s = fma(av[u][k], bv[u][k], s);
+                }
+            }
+    }
+    return s;
+}
+
+// The same on any basis: a warp per block.
+template <int KIND>
+__device__ double sum_mixed(const RedItem &it, const int32_t *nb, int64_t b0, int64_t b1)
+{
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int64_t b = b0 + (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5); b < b1;
+         b += (int64_t)gridDim.x * (RED_T / 32)) {
+        const int i = it.row[b], j = it.col[b];
+        const int ni = nb[i], nj = nb[j];
+        const double *a = it.A + it.a_off[b];
+        const double *bb = it.B;
+        if (KIND == RED_TRACE) {
+            const int64_t t = it.bmap[b];
+            if (t < 0) continue;
+            bb += it.b_off[t];
+        } else if (KIND == RED_DOT) {
+            bb += it.a_off[b];
+        }
+        for (int e = lane; e < ni * nj; e += 32) {
+            if (KIND == RED_TRACE) {
+                const int r = e / nj, q = e - r * nj;
+                s = fma(a[e], bb[q * ni + r], s);
+            } else if (KIND == RED_DOT) {
+                s = fma(a[e], bb[e], s);
+            } else {
+                double v = a[e];
+                if (i == j && (e / nj) == (e % nj)) v -= 1.0;
+                s = fma(v, v, s);
+            }
+        }
+    }
+    return s;
+}
+
+template <int KIND, int NB>
+__device__ __forceinline__ double sum_of(const RedItem &it, const int32_t *nb, int64_t b0,
+                                         int64_t b1)
+{
+    if constexpr (NB != 0) return sum_uniform<KIND, NB>(it, b0, b1);
+    else return sum_mixed<KIND>(it, nb, b0, b1);
+}
+
+// Quantity blockIdx.z of cell blockIdx.y, NB orbitals per atom (0: any).
+template <int NB>
+__global__ void __launch_bounds__(RED_T, 3) k_reduce(const __grid_constant__ RedArgs a)
+{
+    const RedItem &it = a.it[blockIdx.z];
+    const int64_t unit = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
+    const int64_t b0 = it.seg ? it.seg[blockIdx.y] : 0;
+    const int64_t b1 = it.seg ? it.seg[blockIdx.y + 1] : it.nblk;
+    double s;
+    if (it.kind == RED_TRACE)
+        s = sum_of<RED_TRACE, NB>(it, a.nb, b0, b1);
+    else if (it.kind == RED_DOT)
+        s = sum_of<RED_DOT, NB>(it, a.nb, b0, b1);
+    else
+        s = sum_of<RED_FROB_MI, NB>(it, a.nb, b0, b1);
+    s = cta_reduce<SUM>(s);
+    double *part = a.sink.part + unit * gridDim.x;
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    if (!last_arrival(a.sink, unit)) return;
+    s = fold<SUM>(part, 1);
+    if (threadIdx.x == 0) {
+        a.sink.out[unit] = s;
+        if (unit == 0) publish_flag(a.sink);
+    }
+}
+
+// Gershgorin data per scalar row: 32 / n_i atom rows per warp (two on a mixed basis), one lane
+// per scalar row, which adds its values in the order of the columns (the sums are those of a
+// plain loop to the bit).  Bound by the FP64 pipe (an add occupies it 16 clocks a warp) and by
+// latency: the values of the next three 9-orbital blocks (six of 4 orbitals, one of a mixed
+// basis) are fetched under the sums of these, and the first warps of all CTAs get work before
+// the second ones do.  S of 216 atoms: 166 us with a warp per row and a plain loop, 128 with
+// the prefetch on 27 CTAs, some 60 spread over 72.
+template <int NB>
+__global__ void __launch_bounds__(RED_T)
+k_row_bounds(int n_atoms, const int32_t *cell_start, const int64_t *rp, const int32_t *col,
+             const int32_t *nb, const int64_t *off, const double *M, const RedSink sink)
+{
+    constexpr int W = NB ? NB : 16, U = NB ? 27 / NB : 1, ST = (NB * NB + 1) & ~1, PER = 32 / W;
+    const int sub = (threadIdx.x & 31) / W, lane = (threadIdx.x & 31) % W;
+    const int i1 = cell_start ? cell_start[blockIdx.y + 1] : n_atoms;
+    double lo = DBL_MAX, hi = -DBL_MAX, amax = 0.0;
+    for (int i = (cell_start ? cell_start[blockIdx.y] : 0) +
+                 PER * (blockIdx.x + gridDim.x * (threadIdx.x >> 5)) + sub;
+         i < i1 && sub < PER; i += PER * gridDim.x * (RED_T / 32)) {
+        const int ni = NB ? NB : nb[i];
+        if (lane >= ni) continue;
+        const int64_t b1 = rp[i + 1];
+        double v[U][W], w[U][W];
+        int j[U], nj[U], jw[U], njw[U];  // column atom, its orbitals (0 past the row's end)
+        auto load = [&](int64_t b, double (&x)[U][W], int (&jx)[U], int (&nx)[U]) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool ok = b + u < b1;
+                jx[u] = ok ? __ldg(col + b + u) : -1;
+                nx[u] = !ok ? 0 : NB ? NB : __ldg(nb + jx[u]);
+                const double *m = M + (!ok ? 0 : (NB ? (b + u) * ST : __ldg(off + b + u)) +
+                                                     lane * nx[u]);
+#pragma unroll
+                for (int q = 0; q < W; ++q) x[u][q] = q < nx[u] ? __ldg(m + q) : 0.0;
+            }
+        };
+        double centre = 0.0, rad = 0.0, tot = 0.0;
+        int64_t b = rp[i];
+        load(b, v, j, nj);
+        while (b < b1) {
+            b += U;
+            load(b, w, jw, njw);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < W; ++q) {
+                    if (q < nj[u]) {
+                        tot += fabs(v[u][q]);
+                        if (j[u] == i && q == lane)
+                            centre = v[u][q];
+                        else
+                            rad += fabs(v[u][q]);
+                    }
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                j[u] = jw[u];
+                nj[u] = njw[u];
+#pragma unroll
+                for (int q = 0; q < W; ++q) v[u][q] = w[u][q];
             }
         }
         lo = fmin(lo, centre - rad);
@@ -153,18 +314,32 @@ k_row_bounds(int n_atoms, const int64_t *rp, const int32_t *col, const int32_t *
     lo = cta_reduce<MIN>(lo);
     hi = cta_reduce<MAX>(hi);
     amax = cta_reduce<MAX>(amax);
+    double *part = sink.part + 3 * (int64_t)blockIdx.y * gridDim.x;
     if (threadIdx.x == 0) {
         part[3 * blockIdx.x + 0] = lo;
         part[3 * blockIdx.x + 1] = hi;
         part[3 * blockIdx.x + 2] = amax;
     }
+    if (!last_arrival(sink, blockIdx.y)) return;
+    lo = fold<MIN>(part + 0, 3);
+    hi = fold<MAX>(part + 1, 3);
+    amax = fold<MAX>(part + 2, 3);
+    if (threadIdx.x == 0) {
+        double *o = sink.out + 3 * blockIdx.y;
+        o[0] = lo;
+        o[1] = hi;
+        o[2] = amax;
+        if (blockIdx.y == 0) publish_flag(sink);
+    }
 }
 
-__global__ void k_axpby(int64_t n, double a, const double *x, double b, double *y)
+// y <- a x + b z (y may be x or z; b == 0: z not read)
+__global__ void k_lincomb(int64_t n, double a, const double *x, double b, const double *z,
+                          double *y)
 {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x)
-        y[e] = (b == 0.0) ? a * x[e] : a * x[e] + b * y[e];
+        y[e] = (b == 0.0) ? a * x[e] : a * x[e] + b * z[e];
 }
 
 // dst_b = s * (src_ij or src_ji^T) + bb * dst_b; warp per destination block.
@@ -206,30 +381,6 @@ __global__ void k_identity(int n_atoms, const int64_t *rp, const int32_t *col,
     for (int r = 0; r < ni; ++r) M[off[lo] + r * ni + r] = s;
 }
 
-// G_E = 2[3(Z + Z^T) - 2((R1 + R1^T) + R2)], G_N = 12(U - R3) on P_L (warp per L block).
-__global__ void k_lnv_grad(int64_t nblk, const int32_t *row, const int32_t *col,
-                           const int32_t *nb, const int64_t *l_off, const int64_t *l_tr,
-                           const int64_t *u_off, const int64_t *map_u, const int64_t *map_ut,
-                           const double *Z, const double *U, const double *R1,
-                           const double *R2, const double *R3, double *GE, double *GN)
-{
-    const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (b >= nblk) return;
-    const int ni = nb[row[b]], nj = nb[col[b]];
-    const int64_t lb = l_off[b], lt = l_off[l_tr[b]];
-    const int64_t zb = map_u[b], zt = map_ut[b];
-    for (int e = lane; e < ni * nj; e += 32) {
-        const int r = e / nj, q = e - r * nj;
-        const double z = zb >= 0 ? Z[u_off[zb] + e] : 0.0;
-        const double zT = zt >= 0 ? Z[u_off[zt] + q * ni + r] : 0.0;
-        const double u = zb >= 0 ? U[u_off[zb] + e] : 0.0;
-        const double t = (R1[lb + e] + R1[lt + q * ni + r]) + R2[lb + e];
-        GE[lb + e] = 2.0 * (3.0 * (z + zT) - 2.0 * t);
-        GN[lb + e] = 12.0 * (u - R3[lb + e]);
-    }
-}
-
 __global__ void k_lnv_grad_n(int64_t nblk, const int32_t *row, const int32_t *col,
                              const int32_t *nb, const int64_t *l_off, const int64_t *u_off,
                              const int64_t *map_u, const double *U, const double *R3,
@@ -266,109 +417,17 @@ __global__ void k_lnv_grad_e(int64_t nblk, const int32_t *row, const int32_t *co
     }
 }
 
-// ---------------- per-cell (segmented) versions: blockIdx.y = cell, RED_S CTAs per cell
-constexpr int RED_S = 64;
+// ---------------- per-cell versions: blockIdx.y = cell
 
-__global__ void __launch_bounds__(RED_T)
-k_trace_seg(const int64_t *seg, const int32_t *row, const int32_t *col, const int32_t *nb,
-            const int64_t *a_off, const int64_t *b_off, const int64_t *bmap, const double *A,
-            const double *B, double *part)
-{
-    const int lane = threadIdx.x & 31, c = blockIdx.y;
-    const int64_t b0 = seg[c], b1 = seg[c + 1];
-    double s = 0.0;
-    for (int64_t b = b0 + (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5); b < b1;
-         b += (int64_t)RED_S * (RED_T / 32)) {
-        const int64_t t = bmap[b];
-        if (t < 0) continue;
-        const int ni = nb[row[b]], nj = nb[col[b]];
-        const double *a = A + a_off[b];
-        const double *bb = B + b_off[t];
-        for (int e = lane; e < ni * nj; e += 32) {
-            const int r = e / nj, q = e - r * nj;
-            s = fma(a[e], bb[q * ni + r], s);
-        }
-    }
-    s = cta_reduce<SUM>(s);
-    if (threadIdx.x == 0) part[(int64_t)c * RED_S + blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(RED_T)
-k_dot_seg(const int64_t *seg, const int32_t *row, const int32_t *col, const int32_t *nb,
-          const int64_t *off, const double *A, const double *B, double *part)
-{
-    const int lane = threadIdx.x & 31, c = blockIdx.y;
-    const int64_t b0 = seg[c], b1 = seg[c + 1];
-    double s = 0.0;
-    for (int64_t b = b0 + (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5); b < b1;
-         b += (int64_t)RED_S * (RED_T / 32)) {
-        const int sz = nb[row[b]] * nb[col[b]];
-        const int64_t o = off[b];
-        for (int e = lane; e < sz; e += 32) s = fma(A[o + e], B[o + e], s);
-    }
-    s = cta_reduce<SUM>(s);
-    if (threadIdx.x == 0) part[(int64_t)c * RED_S + blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(RED_T)
-k_row_bounds_seg(const int32_t *cell_start, const int64_t *rp, const int32_t *col,
-                 const int32_t *nb, const int64_t *off, const double *M, double *part)
-{
-    const int lane = threadIdx.x & 31, c = blockIdx.y;
-    double lo = DBL_MAX, hi = -DBL_MAX, amax = 0.0;
-    for (int i = cell_start[c] + blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5);
-         i < cell_start[c + 1]; i += RED_S * (RED_T / 32)) {
-        const int ni = nb[i];
-        if (lane >= ni) continue;
-        double centre = 0.0, rad = 0.0, tot = 0.0;
-        for (int64_t b = rp[i]; b < rp[i + 1]; ++b) {
-            const int j = col[b], nj = nb[j];
-            const double *m = M + off[b] + (int64_t)lane * nj;
-            for (int q = 0; q < nj; ++q) {
-                const double v = m[q];
-                tot += fabs(v);
-                if (j == i && q == lane)
-                    centre = v;
-                else
-                    rad += fabs(v);
-            }
-        }
-        lo = fmin(lo, centre - rad);
-        hi = fmax(hi, centre + rad);
-        amax = fmax(amax, tot);
-    }
-    lo = cta_reduce<MIN>(lo);
-    hi = cta_reduce<MAX>(hi);
-    amax = cta_reduce<MAX>(amax);
-    if (threadIdx.x == 0) {
-        const int64_t k = (int64_t)c * RED_S + blockIdx.x;
-        part[3 * k + 0] = lo;
-        part[3 * k + 1] = hi;
-        part[3 * k + 2] = amax;
-    }
-}
-
-// one CTA per cell folds that cell's RED_S partials (strided) into out[cell * ostride]
-template <int OP>
-__global__ void k_final_seg(const double *part, int stride, double *out, int ostride)
-{
-    const int c = blockIdx.x;
-    double v = identity_of<OP>();
-    for (int e = threadIdx.x; e < RED_S; e += RED_T)
-        v = combine<OP>(v, part[((int64_t)c * RED_S + e) * stride]);
-    v = cta_reduce<OP>(v);
-    if (threadIdx.x == 0) out[(int64_t)c * ostride] = v;
-}
-
-__global__ void k_axpby_seg(const int64_t *seg_val, const double *coef, int n_cells,
-                            const double *x, double *y)
+__global__ void k_lincomb_seg(const int64_t *seg_val, const double *coef, int n_cells,
+                              const double *x, const double *z, double *y)
 {
     const int c = blockIdx.y;
     const double a = coef[c], b = coef[n_cells + c];
     const int64_t v1 = seg_val[c + 1];
     for (int64_t e = seg_val[c] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < v1;
          e += (int64_t)gridDim.x * blockDim.x)
-        y[e] = (b == 0.0) ? a * x[e] : a * x[e] + b * y[e];
+        y[e] = (b == 0.0) ? a * x[e] : a * x[e] + b * z[e];
 }
 
 __global__ void k_identity_seg(int n_atoms, const int32_t *cell_of, const int64_t *rp,
@@ -390,86 +449,93 @@ __global__ void k_identity_seg(int n_atoms, const int32_t *cell_of, const int64_
     for (int r = 0; r < ni; ++r) M[off[lo] + r * ni + r] = s;
 }
 
-cq_status red_part(cq_ctx *ctx, double **part)
+// Sink of a reduction over `cells` units per quantity whose scalars start at `slot`, and the
+// CTAs of a unit with `work` CTAs' worth of items.
+cq_status red_sink(cq_ctx *ctx, int cells, int64_t work, int slot, RedSink *k, unsigned *ctas)
 {
+    const int64_t cap = std::max(RED_CELL, RED_G / cells);
     void *p;
-    cq_status st = cq_scratch(ctx, "red_part", sizeof(double) * 3 * RED_G, &p);
-    *part = (double *)p;
+    cq_status st = cq_scratch(ctx, "red_part", sizeof(double) * RED_Q * cap * cells, &p);
+    k->part = (double *)p;
+    k->count = ctx->red_count.as<uint32_t>();
+    k->out = ctx->host_out + slot;
+    k->flag = ctx->flag.as<int32_t>();
+    k->flag_out = reinterpret_cast<int32_t *>(ctx->host_out + CQ_RED_SLOTS - 1);
+    *ctas = (unsigned)std::min(cap, std::max<int64_t>(1, work));
     return st;
 }
 
 }  // namespace
 
-cq_status cq_trace_dev(cq_ctx *ctx, const cq_pattern *pA, const double *A,
-                       const cq_pattern *pB, const double *B, int slot)
+cq_status cq_reduce(cq_ctx *ctx, int nq, const RedQ *q, bool per_cell, int slot)
 {
-    const int64_t *bmap;
-    cq_status st = cq_get_map(ctx, pB, pA, 1, &bmap);
+    const int nc = per_cell ? q[0].pA->n_cells() : 1;
+    const int nbu = q[0].pA->geo->uniform_nb;
+    RedArgs a = {};
+    int64_t nblk = 0;
+    for (int e = 0; e < nq; ++e) {
+        RedItem &it = a.it[e];
+        const cq_pattern *pA = q[e].pA;
+        it.kind = q[e].kind;
+        it.nblk = pA->n_blocks;
+        it.seg = nc > 1 ? pA->seg_blk_dev.as<int64_t>() : nullptr;
+        it.a_off = pA->val_off.as<int64_t>();
+        it.row = pA->row.as<int32_t>();
+        it.col = pA->col.as<int32_t>();
+        it.A = q[e].A;
+        it.B = q[e].B;
+        if (it.kind == RED_TRACE) {
+            cq_status st = cq_get_map(ctx, q[e].pB, pA, 1, &it.bmap);
+            if (st != CQ_OK) return st;
+            it.b_off = q[e].pB->val_off.as<int64_t>();
+        }
+        nblk = std::max(nblk, it.nblk);
+    }
+    a.nb = q[0].pA->geo->nb.as<int32_t>();
+    unsigned ctas;
+    // a CTA takes 32 blocks (64 of 4 orbitals) at a time
+    cq_status st = red_sink(ctx, nc, (nblk / nc + 31) / 32, slot, &a.sink, &ctas);
     if (st != CQ_OK) return st;
-    double *part;
-    if ((st = red_part(ctx, &part)) != CQ_OK) return st;
-    k_trace<<<RED_G, RED_T, 0, ctx->stream>>>(pA->n_blocks, pA->row.as<int32_t>(),
-                                              pA->col.as<int32_t>(), pA->geo->nb.as<int32_t>(),
-                                              pA->val_off.as<int64_t>(), pB->val_off.as<int64_t>(),
-                                              bmap, A, B, part);
-    k_final<SUM><<<1, RED_T, 0, ctx->stream>>>(part, RED_G, 1, ctx->red_out.as<double>() + slot);
-    cq_count_launch(2);
-    return cq_check_cuda(ctx, cudaGetLastError(), "trace");
+    const dim3 grid(ctas, (unsigned)nc, (unsigned)nq);
+    if (nbu == 9)
+        k_reduce<9><<<grid, RED_T, 0, ctx->stream>>>(a);
+    else if (nbu == 4)
+        k_reduce<4><<<grid, RED_T, 0, ctx->stream>>>(a);
+    else
+        k_reduce<0><<<grid, RED_T, 0, ctx->stream>>>(a);
+    cq_count_launch();
+    return cq_check_cuda(ctx, cudaGetLastError(), "reduction");
 }
 
-cq_status cq_dot_dev(cq_ctx *ctx, const cq_pattern *p, const double *A, const double *B,
-                     int slot)
+cq_status cq_row_bounds_dev(cq_ctx *ctx, const cq_pattern *p, const double *M, bool per_cell,
+                            int slot)
 {
-    double *part;
-    cq_status st = red_part(ctx, &part);
+    const int nc = per_cell ? p->n_cells() : 1;
+    const int nbu = p->geo->uniform_nb;
+    const int per = nbu == 9 ? 3 : nbu == 4 ? 8 : 2;  // atom rows of a warp
+    RedSink sink;
+    unsigned ctas;
+    cq_status st = red_sink(ctx, nc, (p->geo->n_atoms / nc + per - 1) / per, slot, &sink, &ctas);
     if (st != CQ_OK) return st;
-    k_dot<<<RED_G, RED_T, 0, ctx->stream>>>(p->n_blocks, p->row.as<int32_t>(),
-                                            p->col.as<int32_t>(), p->geo->nb.as<int32_t>(),
-                                            p->val_off.as<int64_t>(), A, B, part);
-    k_final<SUM><<<1, RED_T, 0, ctx->stream>>>(part, RED_G, 1, ctx->red_out.as<double>() + slot);
-    cq_count_launch(2);
-    return cq_check_cuda(ctx, cudaGetLastError(), "dot");
-}
-
-cq_status cq_frob2_minus_identity_dev(cq_ctx *ctx, const cq_pattern *p, const double *M,
-                                      int slot)
-{
-    double *part;
-    cq_status st = red_part(ctx, &part);
-    if (st != CQ_OK) return st;
-    k_frob2_mi<<<RED_G, RED_T, 0, ctx->stream>>>(p->n_blocks, p->row.as<int32_t>(),
-                                                 p->col.as<int32_t>(), p->geo->nb.as<int32_t>(),
-                                                 p->val_off.as<int64_t>(), M, part);
-    k_final<SUM><<<1, RED_T, 0, ctx->stream>>>(part, RED_G, 1, ctx->red_out.as<double>() + slot);
-    cq_count_launch(2);
-    return cq_check_cuda(ctx, cudaGetLastError(), "frob2");
-}
-
-cq_status cq_row_bounds_dev(cq_ctx *ctx, const cq_pattern *p, const double *M, int slot)
-{
-    double *part;
-    cq_status st = red_part(ctx, &part);
-    if (st != CQ_OK) return st;
-    k_row_bounds<<<RED_G, RED_T, 0, ctx->stream>>>(p->geo->n_atoms, p->row_ptr.as<int64_t>(),
-                                                   p->col.as<int32_t>(), p->geo->nb.as<int32_t>(),
-                                                   p->val_off.as<int64_t>(), M, part);
-    double *o = ctx->red_out.as<double>() + slot;
-    k_final<MIN><<<1, RED_T, 0, ctx->stream>>>(part + 0, RED_G, 3, o + 0);
-    k_final<MAX><<<1, RED_T, 0, ctx->stream>>>(part + 1, RED_G, 3, o + 1);
-    k_final<MAX><<<1, RED_T, 0, ctx->stream>>>(part + 2, RED_G, 3, o + 2);
-    cq_count_launch(4);
+    auto kernel = nbu == 9 ? k_row_bounds<9> : nbu == 4 ? k_row_bounds<4> : k_row_bounds<0>;
+    kernel<<<dim3(ctas, (unsigned)nc), RED_T, 0, ctx->stream>>>(
+        p->geo->n_atoms, nc > 1 ? p->geo->cell_start_dev.as<int32_t>() : nullptr,
+        p->row_ptr.as<int64_t>(), p->col.as<int32_t>(), p->geo->nb.as<int32_t>(),
+        p->val_off.as<int64_t>(), M, sink);
+    cq_count_launch();
     return cq_check_cuda(ctx, cudaGetLastError(), "row bounds");
 }
 
-cq_status cq_axpby(cq_ctx *ctx, int64_t n, double a, const double *x, double b, double *y)
+cq_status cq_lincomb(cq_ctx *ctx, int64_t n, double a, const double *x, double b, const double *z,
+                     double *y)
 {
     if (n == 0) return CQ_OK;
     int64_t blocks = (n + 255) / 256;
     const int64_t cap = (int64_t)ctx->num_sms * 16;
     if (blocks > cap) blocks = cap;
-    k_axpby<<<(unsigned)blocks, 256, 0, ctx->stream>>>(n, a, x, b, y);
+    k_lincomb<<<(unsigned)blocks, 256, 0, ctx->stream>>>(n, a, x, b, z, y);
     cq_count_launch();
-    return cq_check_cuda(ctx, cudaGetLastError(), "axpby");
+    return cq_check_cuda(ctx, cudaGetLastError(), "lincomb");
 }
 
 cq_status cq_gather(cq_ctx *ctx, const cq_pattern *pSrc, const double *src,
@@ -501,85 +567,10 @@ cq_status cq_set_identity(cq_ctx *ctx, const cq_pattern *p, double *M, double s)
     return cq_check_cuda(ctx, cudaGetLastError(), "identity");
 }
 
-cq_status cq_lnv_gradients(cq_ctx *ctx, const cq_pattern *pL, const cq_pattern *pU,
-                           const double *Z, const double *U, const double *R1,
-                           const double *R2, const double *R3, double *GE, double *GN)
-{
-    const int64_t *mu, *mut;
-    cq_status st = cq_get_map(ctx, pU, pL, 0, &mu);
-    if (st != CQ_OK) return st;
-    if ((st = cq_get_map(ctx, pU, pL, 1, &mut)) != CQ_OK) return st;
-    if (pL->n_blocks == 0) return CQ_OK;
-    k_lnv_grad<<<(unsigned)((pL->n_blocks + 7) / 8), 256, 0, ctx->stream>>>(
-        pL->n_blocks, pL->row.as<int32_t>(), pL->col.as<int32_t>(), pL->geo->nb.as<int32_t>(),
-        pL->val_off.as<int64_t>(), pL->transpose.as<int64_t>(), pU->val_off.as<int64_t>(), mu, mut,
-        Z, U, R1, R2, R3, GE, GN);
-    cq_count_launch();
-    return cq_check_cuda(ctx, cudaGetLastError(), "lnv gradients");
-}
-
 // ---------------------------------------------------------------- per-cell host wrappers
 
-static cq_status seg_part(cq_ctx *ctx, int n_cells, double **part)
-{
-    void *p;
-    cq_status st = cq_scratch(ctx, "red_part_seg", sizeof(double) * 3 * RED_S * n_cells, &p);
-    *part = (double *)p;
-    return st;
-}
-
-cq_status cq_trace_seg_dev(cq_ctx *ctx, const cq_pattern *pA, const double *A,
-                           const cq_pattern *pB, const double *B, int slot)
-{
-    const int64_t *bmap;
-    cq_status st = cq_get_map(ctx, pB, pA, 1, &bmap);
-    if (st != CQ_OK) return st;
-    const int nc = pA->n_cells();
-    double *part;
-    if ((st = seg_part(ctx, nc, &part)) != CQ_OK) return st;
-    k_trace_seg<<<dim3(RED_S, nc), RED_T, 0, ctx->stream>>>(
-        pA->seg_blk_dev.as<int64_t>(), pA->row.as<int32_t>(), pA->col.as<int32_t>(),
-        pA->geo->nb.as<int32_t>(), pA->val_off.as<int64_t>(), pB->val_off.as<int64_t>(), bmap, A,
-        B, part);
-    k_final_seg<SUM><<<nc, RED_T, 0, ctx->stream>>>(part, 1, ctx->red_out.as<double>() + slot, 1);
-    cq_count_launch(2);
-    return cq_check_cuda(ctx, cudaGetLastError(), "trace (cells)");
-}
-
-cq_status cq_dot_seg_dev(cq_ctx *ctx, const cq_pattern *p, const double *A, const double *B,
-                         int slot)
-{
-    const int nc = p->n_cells();
-    double *part;
-    cq_status st = seg_part(ctx, nc, &part);
-    if (st != CQ_OK) return st;
-    k_dot_seg<<<dim3(RED_S, nc), RED_T, 0, ctx->stream>>>(
-        p->seg_blk_dev.as<int64_t>(), p->row.as<int32_t>(), p->col.as<int32_t>(),
-        p->geo->nb.as<int32_t>(), p->val_off.as<int64_t>(), A, B, part);
-    k_final_seg<SUM><<<nc, RED_T, 0, ctx->stream>>>(part, 1, ctx->red_out.as<double>() + slot, 1);
-    cq_count_launch(2);
-    return cq_check_cuda(ctx, cudaGetLastError(), "dot (cells)");
-}
-
-cq_status cq_row_bounds_seg_dev(cq_ctx *ctx, const cq_pattern *p, const double *M, int slot)
-{
-    const int nc = p->n_cells();
-    double *part;
-    cq_status st = seg_part(ctx, nc, &part);
-    if (st != CQ_OK) return st;
-    k_row_bounds_seg<<<dim3(RED_S, nc), RED_T, 0, ctx->stream>>>(
-        p->geo->cell_start_dev.as<int32_t>(), p->row_ptr.as<int64_t>(), p->col.as<int32_t>(),
-        p->geo->nb.as<int32_t>(), p->val_off.as<int64_t>(), M, part);
-    double *o = ctx->red_out.as<double>() + slot;
-    k_final_seg<MIN><<<nc, RED_T, 0, ctx->stream>>>(part + 0, 3, o + 0, 3);
-    k_final_seg<MAX><<<nc, RED_T, 0, ctx->stream>>>(part + 1, 3, o + 1, 3);
-    k_final_seg<MAX><<<nc, RED_T, 0, ctx->stream>>>(part + 2, 3, o + 2, 3);
-    cq_count_launch(4);
-    return cq_check_cuda(ctx, cudaGetLastError(), "row bounds (cells)");
-}
-
-cq_status cq_axpby_seg(cq_ctx *ctx, const cq_pattern *p, const double *a, const double *x,
-                       const double *b, double *y)
+cq_status cq_lincomb_seg(cq_ctx *ctx, const cq_pattern *p, const double *a, const double *x,
+                         const double *b, const double *z, double *y)
 {
     const int nc = p->n_cells();
     void *v;
@@ -588,10 +579,10 @@ cq_status cq_axpby_seg(cq_ctx *ctx, const cq_pattern *p, const double *a, const 
     std::vector<double> coef(a, a + nc);
     coef.insert(coef.end(), b, b + nc);
     cudaMemcpyAsync(v, coef.data(), sizeof(double) * 2 * nc, cudaMemcpyHostToDevice, ctx->stream);
-    k_axpby_seg<<<dim3(64, nc), 256, 0, ctx->stream>>>(p->seg_val_dev.as<int64_t>(), (double *)v,
-                                                       nc, x, y);
+    k_lincomb_seg<<<dim3(64, nc), 256, 0, ctx->stream>>>(p->seg_val_dev.as<int64_t>(), (double *)v,
+                                                         nc, x, z, y);
     cq_count_launch();
-    return cq_check_cuda(ctx, cudaGetLastError(), "axpby (cells)");
+    return cq_check_cuda(ctx, cudaGetLastError(), "lincomb (cells)");
 }
 
 cq_status cq_set_identity_seg(cq_ctx *ctx, const cq_pattern *p, double *M, const double *s)
