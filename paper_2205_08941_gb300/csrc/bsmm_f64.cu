@@ -11,10 +11,15 @@
 
 namespace {
 
+// Threads per CTA: nothing is shared beyond the rows of a C block, and small CTAs fill the last
+// wave better (U.X on 64 atoms: 32.9 us with 64 threads, 37.0 with 256 at the same lane split;
+// large products do not change).
+constexpr int F64_T = 64;
+
 // One or two products over the same task list (blockIdx.y picks the operands): the pairs of an
 // LNV evaluation that share their patterns go in one launch.  A 64-atom cell's product is one
 // wave of short dependent chains (22 us alone), so its partner runs beside it for little: an
-// LNV step at 64 atoms takes 6.3 ms (7.4 ms with one product per launch and 16 lanes per row).
+// LNV run at 64 atoms takes 6.3 ms (7.4 ms with one product per launch and 16 lanes per row).
 struct F64Ops {
     const double *A[2], *B[2];
     double *C[2];
@@ -25,7 +30,7 @@ struct F64Ops {
 // FMAs in the same order).  Large products are FP64-bound and do not change; with 4 orbitals
 // and 64 atoms U.X goes from 39 to 37 us.
 template <int NB, int Q, bool VEC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(F64_T)
 k_bsmm_f64_uniform(int64_t n_items, const int64_t *__restrict__ seg,
                    const int2 *__restrict__ tasks, const F64Ops ops, int stride, double alpha,
                    double beta)
@@ -154,7 +159,7 @@ __device__ __forceinline__ void generic_row(unsigned gmask, int q, int64_t c, in
 // four cells of 5/9/13 orbitals: 56.5 ms unsorted at q = 8, 45.0 with sorted tasks, 33.1 with
 // both at q = 4; U.X 76.7 -> 50.2 ms, 0.97 of the pipe's 1.26 TFLOP/s).
 template <int Q>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(F64_T)
 k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ rowitem,
                    const int32_t *__restrict__ order,
                    const int64_t *__restrict__ seg, const int2 *__restrict__ tasks,
@@ -170,7 +175,7 @@ k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ row
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t item = gt / Q;
     const int q = (int)(gt % Q);
-    // the block of the CTA's first item, then each thread's among the next 256 / Q
+    // the block of the CTA's first item, then each thread's among the next F64_T / Q
     __shared__ int64_t first;
     if (threadIdx.x < 32) {
         const int64_t i0 = (int64_t)blockIdx.x * (blockDim.x / Q);
@@ -216,13 +221,16 @@ k_bsmm_f64_generic(int64_t n_items, int64_t n_c, const int64_t *__restrict__ row
 // touches about q cache lines: at q = 16 and 32 the L1 serves one line per clock and the kernel
 // runs at 0.6 of the FP64 pipe (T.V on 216 SZP atoms: 4.02 ms at q = 4, 8.19 at 16); at q = 1
 // short segments end at different times (L.S on 512 atoms: 8.58 ms at q = 4, 9.94 at 1).  So four
-// lanes, two on a 4-orbital basis (S.X on 512 sp atoms: 719 us at 2, 782 at 4), and up to eight
-// while the launch is small (less than 100 k threads) and a lane keeps four tasks, or is tiny.
+// lanes, two on a 4-orbital basis (S.X on 512 sp atoms: 719 us at 2, 782 at 4).  Up to eight
+// lanes where that still leaves less than 60 k threads, so that the SMs have warps to switch
+// between (4 orbitals, U.X on 64 atoms: 32.8 us at 2, 29.0 at 4, 34.8 at 8; on 32 atoms 18.3, 12.2
+// and 11.0), or less than 200 k if segments are long (U.X on 216 atoms: 264 us at 2, 246 at 4).
 int pick_q(const TaskList *tl, int nb)
 {
     const double avg = tl->n_c ? (double)tl->n_tasks / (double)tl->n_c : 0.0;
     int q = nb == 4 ? 2 : 4;
-    while (q < 8 && tl->n_items * q < 100000 && (avg >= 8.0 * q || tl->n_items * q < 8000)) q <<= 1;
+    while (q < 8 && (tl->n_items * q < 30000 || (tl->n_items * q < 100000 && avg >= 64.0 * q)))
+        q <<= 1;
     return q;
 }
 
@@ -233,7 +241,7 @@ void launch_uniform(int q, dim3 grid, cudaStream_t s, int64_t n_items, const Tas
     const int64_t *seg = tl->seg.as<int64_t>();
     const int2 *tk = tl->tasks.as<int2>();
 #define CQ_LAUNCH(QQ) \
-    k_bsmm_f64_uniform<NB, QQ, VEC><<<grid, 256, 0, s>>>(n_items, seg, tk, ops, stride, alpha, beta)
+    k_bsmm_f64_uniform<NB, QQ, VEC><<<grid, F64_T, 0, s>>>(n_items, seg, tk, ops, stride, alpha, beta)
     switch (q) {
     case 1: CQ_LAUNCH(1); break;
     case 2: CQ_LAUNCH(2); break;
@@ -255,7 +263,7 @@ static void launch_f64(cq_ctx *ctx, int q, const TaskList *tl, double alpha,
     const int nbu = pC->geo->uniform_nb;
     cudaStream_t s = ctx->stream;
     const int64_t n_items = tl->n_items;
-    const dim3 grid((unsigned)((n_items * q + 255) / 256), (unsigned)n);
+    const dim3 grid((unsigned)((n_items * q + F64_T - 1) / F64_T), (unsigned)n);
     if (nbu == 9 || nbu == 4) {
         uintptr_t bits = 0;
         for (int e = 0; e < n; ++e)
@@ -269,7 +277,7 @@ static void launch_f64(cq_ctx *ctx, int q, const TaskList *tl, double alpha,
     const int64_t *rowitem = tl->c_rowitem.as<int64_t>();
     const int32_t *nb = pC->geo->nb.as<int32_t>();
 #define CQ_GEN(QQ)                                                                            \
-    k_bsmm_f64_generic<QQ><<<grid, 256, 0, s>>>(                                              \
+    k_bsmm_f64_generic<QQ><<<grid, F64_T, 0, s>>>(                                              \
         n_items, tl->n_c, rowitem, tl->c_order.as<int32_t>(), tl->seg.as<int64_t>(),          \
         tl->tasks.as<int2>(), nb, pC->row.as<int32_t>(), pC->col.as<int32_t>(),               \
         pA->col.as<int32_t>(), pA->val_off.as<int64_t>(), pB->val_off.as<int64_t>(),          \
