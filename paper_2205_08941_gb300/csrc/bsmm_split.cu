@@ -341,26 +341,132 @@ k_piece_index(int gsize, int ca, const int32_t *ent_group, const int32_t *ent_ke
     }
 }
 
-// Main pieces of entries [e0, e0 + n) (one thread per (entry, row)), entry = (atom group,
-// K atom k), index = its block per slot (k_piece_index with one atom per key).  A side
-// (LEFT): row r = (slot r / NB, orbital o), K = orbital m < 8 of k: A_ik[o][m]; B side: row
-// r = (slot, orbital o of j), K = m: B_kj[m][o].
-template <int NB, bool LEFT>
-__global__ void __launch_bounds__(256)
-k_pack_main(int64_t e0, int64_t n, const int32_t *index, const double *__restrict__ X,
-            int stride, uint8_t *pieces)
+__device__ __forceinline__ void pack_copy(void *dst, const void *src, bool wide)
 {
-    constexpr int ROWS = LEFT ? MT : NT, G = ROWS / NB, COLB = LEFT ? COLB_A : COLB_B;
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n * ROWS) return;
-    const int64_t el = q / ROWS;
-    const int r = (int)(q % ROWS), o = r % NB;
-    const int64_t b = r < G * NB ? __ldg(&index[(e0 + el) * G + r / NB]) : -1;
-    double x[8];
+    if (wide)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src));
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src));
+}
+
+// Main and tail pieces of 9-orbital atoms: a CTA (one thread per row) per tail entry (atom group
+// g, tail group tau) makes that tail piece and the main pieces of g with the K atoms of tau,
+// which are consecutive in the main list.  A main entry (g, k): row r = (slot r / 9, orbital
+// o), K = orbital m < 8 of k, index = its block per slot; A side (LEFT): A_ik[o][m], B side
+// (o of j): B_kj[m][o].  Orbital 8 of the u-th atom of tau is K position u of the tail piece
+// (two core columns).
+//
+// Bound by HBM (a block's 648 B are read once; a piece's rows are written whether or not the
+// slot has a block).  A warp copies whole blocks into shared
+// memory, the next entry's while this one is split, because a thread that reads its row from
+// global memory takes one load per value 72 bytes from its neighbour's: 18 L1 lines per load,
+// and the ninth column once more in a pass of its own.  U.X on 4096 atoms: U (4.5 GB, 8 GB of
+// pieces at most) 2.53 ms, X 0.99 ms; with row loads and separate tails 2.86 and 1.29 ms.
+// Skipping the conversions of warps without a block changed nothing.
+// VEC: X starts on a 16-byte boundary (as do then all blocks), else 8-byte copies.
+template <bool LEFT, bool VEC>
+__global__ void __launch_bounds__(LEFT ? MT : NT)
+k_pack9(int64_t t0, int64_t m0, const int32_t *t_group, const int32_t *t_key, const int64_t *m_ptr,
+        const int32_t *m_key, const int32_t *m_index, const double *__restrict__ X,
+        uint8_t *main_pieces, uint8_t *tail_pieces)
+{
+    constexpr int ROWS = LEFT ? MT : NT, G = ROWS / 9, COLB = LEFT ? COLB_A : COLB_B, BS = 82;
+    constexpr int TG = KPieces<9>::TG, WARPS = ROWS / 32, SL = (G + WARPS - 1) / WARPS;
+    __shared__ __align__(16) double buf[2][G * BS];
+    __shared__ uint16_t tail[3][TG][ROWS];
+    const int r = threadIdx.x, lane = r & 31, warp = r >> 5, slot = r / 9, o = r % 9;
+    const int64_t te = t0 + blockIdx.x;
+    const int g = t_group[te], k0 = t_key[te] * TG;
+    // first main entry of g with a key of at least k0: 32 probes at a time
+    int64_t e = m_ptr[g], hi = m_ptr[g + 1];
+    const int64_t end = hi;
+    while (e < hi) {
+        const int64_t step = (hi - e + 31) / 32, at = e + step * lane;
+        const int n = __popc(__ballot_sync(0xffffffffu, at < hi && __ldg(m_key + at) < k0));
+        hi = n ? min(hi, e + step * n) : e;
+        if (n) e += step * (n - 1) + 1;
+    }
+    // atom of entry x in tau (TG and more: none), its blocks of this warp's slots and of this row
+    auto atom_of = [&](int64_t x) { return x < end ? __ldg(m_key + x) - k0 : TG; };
+    auto row_block = [&](int64_t x) { return slot < G ? __ldg(m_index + x * G + slot) : -1; };
+    auto slot_block = [&](int64_t x, int k) {
+        return warp + WARPS * k < G ? __ldg(m_index + x * G + warp + WARPS * k) : -1;
+    };
+    auto copy = [&](const int32_t (&blk)[SL], double *dst) {
 #pragma unroll
-    for (int m = 0; m < 8; ++m)
-        x[m] = b < 0 ? 0.0 : (LEFT ? X[b * stride + o * NB + m] : X[b * stride + m * NB + o]);
-    put_row3(pieces + el * (3 * COLB), piece_off(0, COLB, 0, 0, r), COLB, x);
+        for (int k = 0; k < SL; ++k) {
+            if (blk[k] < 0) continue;
+            const double *src = X + (int64_t)blk[k] * BS;
+            double *d = dst + (warp + WARPS * k) * BS;
+            if (VEC) {
+                pack_copy(d + 2 * lane, src + 2 * lane, true);
+                if (lane < BS / 2 - 32) pack_copy(d + 64 + 2 * lane, src + 64 + 2 * lane, true);
+            } else {
+                pack_copy(d + lane, src + lane, false);
+                pack_copy(d + 32 + lane, src + 32 + lane, false);
+                if (lane < 81 - 64) pack_copy(d + 64 + lane, src + 64 + lane, false);
+            }
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < TG; ++u) tail[0][u][r] = tail[1][u][r] = tail[2][u][r] = 0;
+    int32_t blk[SL];
+    int u = atom_of(e), b = -1, bn = -1, un = TG;
+    if (u < TG) {
+        b = row_block(e);
+#pragma unroll
+        for (int k = 0; k < SL; ++k) blk[k] = slot_block(e, k);
+        copy(blk, buf[0]);
+        un = atom_of(e + 1);
+    }
+    asm volatile("cp.async.commit_group;");
+    if (un < TG) {
+        bn = row_block(e + 1);
+#pragma unroll
+        for (int k = 0; k < SL; ++k) blk[k] = slot_block(e + 1, k);
+    }
+    for (int st = 0; u < TG; st ^= 1) {
+        if (un < TG) copy(blk, buf[st ^ 1]);
+        asm volatile("cp.async.commit_group;");
+        const int uf = un < TG ? atom_of(e + 2) : TG;
+        int bf = -1;
+        if (uf < TG) {
+            bf = row_block(e + 2);
+#pragma unroll
+            for (int k = 0; k < SL; ++k) blk[k] = slot_block(e + 2, k);
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        double x[8], x8 = 0.0;
+        const double *row = buf[st] + (slot < G ? slot : 0) * BS;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) x[m] = b < 0 ? 0.0 : LEFT ? row[o * 9 + m] : row[m * 9 + o];
+        if (b >= 0) x8 = LEFT ? row[o * 9 + 8] : row[72 + o];
+        put_row3(main_pieces + (e - m0) * (3 * COLB), piece_off(0, COLB, 0, 0, r), COLB, x);
+        __nv_bfloat16 v0, v1, v2;
+        split3(x8, v0, v1, v2);
+        tail[0][u][r] = __bfloat16_as_ushort(v0);
+        tail[1][u][r] = __bfloat16_as_ushort(v1);
+        tail[2][u][r] = __bfloat16_as_ushort(v2);
+        __syncthreads();  // the buffer may be filled again
+        ++e;
+        u = un;
+        un = uf;
+        b = bn;
+        bn = bf;
+    }
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            uint32_t w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                w[k] = tail[pl][8 * c + 2 * k][r] | (uint32_t)tail[pl][8 * c + 2 * k + 1][r] << 16;
+            *reinterpret_cast<uint4 *>(tail_pieces + blockIdx.x * (int64_t)(6 * COLB) +
+                                       piece_off(pl, 2 * COLB, c, COLB, r)) =
+                make_uint4(w[0], w[1], w[2], w[3]);
+        }
 }
 
 // Tail pieces of entries [e0, e0 + n) (one thread per (entry, row)), entry = (atom group,
@@ -1193,50 +1299,52 @@ cq_status run_split(cq_ctx *ctx, const PiecePlan *pl, const Groups *gr, double a
     }
     auto blocks = [](int64_t n, int rows) { return (unsigned)((n * rows + 255) / 256); };
     const int32_t *nbd = pA->geo->nb.as<int32_t>();
-    // main and tail pieces of entries [e0, e0 + n) of one side (LEFT: A)
-    auto pack = [&](bool left, bool main, int64_t e0, int64_t n, const PieceList &pl_,
-                    const double *X, const cq_pattern *pX, void *out) {
-        if (n <= 0) return;
+    // pieces of main entries [m0, m1) and tail entries [t0, t1) of one side (LEFT: A); both
+    // ranges are those of the same atom groups
+    auto pack = [&](bool left, int64_t m0, int64_t m1, int64_t t0, int64_t t1,
+                    const PieceList &pm, const PieceList &pt, const double *X,
+                    const cq_pattern *pX, void *vm, void *vt) {
         const int rows = left ? MT : NT;
-        if constexpr (NB > 0) {
-            if (left && main)
-                k_pack_main<NB, true><<<blocks(n, rows), 256, 0, s>>>(
-                    e0, n, pl_.index.as<int32_t>(), X, pX->uniform, (uint8_t *)out);
-            else if (left)
-                k_pack_tail<NB, true><<<blocks(n, rows), 256, 0, s>>>(
-                    e0, n, pl_.index.as<int32_t>(), X, pX->uniform, (uint8_t *)out);
-            else if (main)
-                k_pack_main<NB, false><<<blocks(n, rows), 256, 0, s>>>(
-                    e0, n, pl_.index.as<int32_t>(), X, pX->uniform, (uint8_t *)out);
-            else
-                k_pack_tail<NB, false><<<blocks(n, rows), 256, 0, s>>>(
-                    e0, n, pl_.index.as<int32_t>(), X, pX->uniform, (uint8_t *)out);
+        if constexpr (NB == 9) {
+            if (t1 <= t0) return;
+            const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+            auto k = left ? (vec ? k_pack9<true, true> : k_pack9<true, false>)
+                          : (vec ? k_pack9<false, true> : k_pack9<false, false>);
+            k<<<(unsigned)(t1 - t0), rows, 0, s>>>(
+                t0, m0, pt.group.as<int32_t>(), pt.key.as<int32_t>(), pm.ptr.as<int64_t>(),
+                pm.key.as<int32_t>(), pm.index.as<int32_t>(), X, (uint8_t *)vm, (uint8_t *)vt);
+            cq_count_launch();
+        } else if constexpr (NB == 4) {
+            if (t1 <= t0) return;
+            auto k = left ? k_pack_tail<NB, true> : k_pack_tail<NB, false>;
+            k<<<blocks(t1 - t0, rows), 256, 0, s>>>(t0, t1 - t0, pt.index.as<int32_t>(), X,
+                                                    pX->uniform, (uint8_t *)vt);
+            cq_count_launch();
         } else {
             const int32_t *tab = left ? gr->g_row.as<int32_t>() : gr->h_col.as<int32_t>();
             const int64_t *off = pX->val_off.as<int64_t>();
-            if (main) {
+            if (m1 > m0) {
                 auto k = left ? k_pack_main_mixed<true> : k_pack_main_mixed<false>;
-                k<<<blocks(n, rows), 256, 0, s>>>(e0, n, pl_.index.as<int32_t>(),
-                                                  pl_.group.as<int32_t>(), pl_.key.as<int32_t>(),
-                                                  gr->rank_atoms.as<int32_t>(), tab, nbd, off, X,
-                                                  (uint8_t *)out);
-            } else {
+                k<<<blocks(m1 - m0, rows), 256, 0, s>>>(
+                    m0, m1 - m0, pm.index.as<int32_t>(), pm.group.as<int32_t>(),
+                    pm.key.as<int32_t>(), gr->rank_atoms.as<int32_t>(), tab, nbd, off, X,
+                    (uint8_t *)vm);
+                cq_count_launch();
+            }
+            if (t1 > t0) {
                 auto k = left ? k_pack_tail_mixed<true> : k_pack_tail_mixed<false>;
-                k<<<blocks(n, rows), 256, 0, s>>>(e0, n, pl_.index.as<int32_t>(),
-                                                  pl_.group.as<int32_t>(), pl_.key.as<int32_t>(),
-                                                  gr->tg_atoms.as<int32_t>(),
-                                                  gr->tg_map.as<int32_t>(), tab, nbd, off, X,
-                                                  (uint8_t *)out);
+                k<<<blocks(t1 - t0, rows), 256, 0, s>>>(
+                    t0, t1 - t0, pt.index.as<int32_t>(), pt.group.as<int32_t>(),
+                    pt.key.as<int32_t>(), gr->tg_atoms.as<int32_t>(), gr->tg_map.as<int32_t>(),
+                    tab, nbd, off, X, (uint8_t *)vt);
+                cq_count_launch();
             }
         }
-        cq_count_launch();
     };
-    pack(false, true, 0, ps.bm.n(), ps.bm, B, pB, vbm);
-    pack(false, false, 0, ps.bt.n(), ps.bt, B, pB, vbt);
+    pack(false, 0, ps.bm.n(), 0, ps.bt.n(), ps.bm, ps.bt, B, pB, vbm, vbt);
     for (size_t q = 0; q < pl->batches.size(); ++q) {
         const PieceBatch &b = pl->batches[q];
-        pack(true, true, b.am0, b.am1 - b.am0, ps.am, A, pA, vam);
-        pack(true, false, b.at0, b.at1 - b.at0, ps.at, A, pA, vat);
+        pack(true, b.am0, b.am1, b.at0, b.at1, ps.am, ps.at, A, pA, vam, vat);
         SplitArgs a;
         a.n_tiles = b.tile1 - b.tile0;
         a.kstart = pl->kstart.as<int64_t>() + b.tile0;
