@@ -11,7 +11,7 @@
 // Small cells: a two-kernel reduction followed by two 8-byte copies cost 10 us of launches for
 // a few us of work.  With all the sums of an evaluation in one launch and no copies, the
 // reductions of an LNV run of 4 steps at 64 atoms take 53 launches and 0.46 ms (280 launches and
-// 1.4 ms before), and the run 4.5 ms (6.3).
+// 1.4 ms before).
 #include <algorithm>
 #include <cfloat>
 
@@ -20,10 +20,11 @@
 namespace {
 
 constexpr int RED_T = 256;
-// CTAs of a quantity: 3 per SM (what 80 registers a thread allow) for one cell, and at least 48
-// for each cell of a batch
-constexpr int RED_G = 456;
-constexpr int RED_CELL = 48;
+// Partials of a quantity and cell.  The sums are those of this many CTAs of eight warps, warp w
+// taking every (8 RED_G)th block from block w on; a CTA does the work of NV of them (below), and
+// partials without blocks, which would add zeros, are left out.
+constexpr int RED_G = 1024;   // one cell, or the whole of several
+constexpr int RED_CELL = 64;  // each cell of a batch
 
 enum Op { SUM = 0, MIN = 1, MAX = 2 };
 
@@ -69,13 +70,13 @@ struct RedSink {
     int32_t *flag_out;
 };
 
-// True in every thread of the last CTA of (blockIdx.z, blockIdx.y) to get here, after thread 0
-// of each has written its partials.
+// True in every thread of the last CTA of (blockIdx.z, blockIdx.y) to get here; the writers of
+// the CTA's partials have fenced them.
 __device__ bool last_arrival(const RedSink &k, int64_t unit)
 {
     __shared__ int last;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         last = atomicAdd(&k.count[unit], 1u) == gridDim.x - 1;
         if (last) k.count[unit] = 0;
     }
@@ -90,10 +91,10 @@ __device__ __forceinline__ void publish_flag(const RedSink &k)
 }
 
 template <int OP>
-__device__ double fold(const double *part, int stride)
+__device__ double fold(const double *part, int n, int stride)
 {
     double v = identity_of<OP>();
-    for (int e = threadIdx.x; e < (int)gridDim.x; e += RED_T)
+    for (int e = threadIdx.x; e < n; e += RED_T)
         v = combine<OP>(v, __ldcg(part + (int64_t)e * stride));
     return cta_reduce<OP>(v);
 }
@@ -109,33 +110,33 @@ struct RedItem {
 
 struct RedArgs {
     RedItem it[RED_Q];
+    int nv;  // partials of a CTA
     const int32_t *nb;
     RedSink sink;
 };
 
-// One CTA's share of a quantity on a uniform basis of NB orbitals.  Offsets need no index loads
-// (the blocks of a uniform basis lie at a fixed stride) and a lane's elements, transposed ones
-// included, have the same place in every block, so four blocks are in flight at once (24 loads
-// per lane for 9 orbitals); the map of the next four arrives meanwhile.  Bound by HBM:
-// a trace and a dot over 4.5 GB each at 4096 atoms take 0.67 ms, 6.7 TB/s (1.02 and 0.89 ms with
-// a warp walking one block at a time through its index arrays).
-template <int KIND, int NB>
-__device__ double sum_uniform(const RedItem &it, int64_t b0, int64_t b1)
+// One CTA's share of a quantity on a uniform basis of NB orbitals: warp per block, as on any basis,
+// and the same sums to the bit.  Offsets need no index loads (the blocks of a uniform basis lie at
+// a fixed stride) and a lane's elements, transposed ones included, have the same place in every
+// block, so a warp keeps four blocks in flight (24 loads per lane for 9 orbitals) and the map of
+// the next four arrives meanwhile.  Bound by HBM: a trace and a dot over 4.5 GB each at 4096 atoms
+// take 0.73 ms, 6.1 TB/s (1.02 and 0.89 ms with a warp walking one block at a time through its
+// index arrays).
+template <int KIND, int NB, int NV>
+__device__ void sum_uniform(const RedItem &it, int64_t b0, int64_t b1, double (&s)[4])
 {
-    constexpr int E = NB * NB, ST = (E + 1) & ~1, LPB = E >= 32 ? 32 : 16, U = 4;
-    constexpr int EPL = (E + LPB - 1) / LPB;
-    const int sub = threadIdx.x % LPB;
+    constexpr int E = NB * NB, ST = (E + 1) & ~1, U = 4, EPL = (E + 31) / 32;
+    const int sub = threadIdx.x & 31;
     int te[EPL];
 #pragma unroll
     for (int k = 0; k < EPL; ++k) {
-        const int e = sub + k * LPB;
+        const int e = sub + 32 * k;
         te[k] = KIND == RED_TRACE ? (e % NB) * NB + e / NB : e;
     }
-    const int64_t W = (int64_t)gridDim.x * (RED_T / LPB);
+    const int64_t W = (int64_t)gridDim.x * (RED_T / 32);
     const double *__restrict__ A = it.A;
     const double *__restrict__ B = it.B;
-    double s = 0.0;
-    int64_t b = b0 + (int64_t)blockIdx.x * (RED_T / LPB) + threadIdx.x / LPB;
+    int64_t b = b0 + (int64_t)blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5);
     int64_t t[U];
     auto partner = [&](int64_t x) -> int64_t {
         if (x >= b1) return -1;
@@ -151,10 +152,10 @@ __device__ double sum_uniform(const RedItem &it, int64_t b0, int64_t b1)
         for (int u = 0; u < U; ++u)
 #pragma unroll
             for (int k = 0; k < EPL; ++k) {
-                const bool ok = t[u] >= 0 && sub + k * LPB < E;
-                av[u][k] = ok ? __ldg(A + (b + u * W) * ST + sub + k * LPB) : 0.0;
+                const bool ok = t[u] >= 0 && sub + 32 * k < E;
+                av[u][k] = ok ? __ldg(A + (b + u * W) * ST + sub + 32 * k) : 0.0;
                 if (KIND == RED_FROB_MI)
-                    bv[u][k] = ok && t[u] && (sub + k * LPB) % (NB + 1) == 0 ? 1.0 : 0.0;
+                    bv[u][k] = ok && t[u] && (sub + 32 * k) % (NB + 1) == 0 ? 1.0 : 0.0;
                 else
                     bv[u][k] = ok ? __ldg(B + t[u] * ST + te[k]) : 0.0;
             }
@@ -167,13 +168,12 @@ __device__ double sum_uniform(const RedItem &it, int64_t b0, int64_t b1)
             for (int k = 0; k < EPL; ++k) {
                 if (KIND == RED_FROB_MI) {
                     const double v = av[u][k] - bv[u][k];
-                    s = fma(v, v, s);
+                    s[u % NV] = fma(v, v, s[u % NV]);
                 } else {
-                    s = fma(av[u][k], bv[u][k], s);
+                    s[u % NV] = fma(av[u][k], bv[u][k], s[u % NV]);
                 }
             }
     }
-    return s;
 }
 
 // The same on any basis: a warp per block.
@@ -211,36 +211,63 @@ __device__ double sum_mixed(const RedItem &it, const int32_t *nb, int64_t b0, in
     return s;
 }
 
+// The sums s[0 .. nv) of the CTA's nv partials: partial i takes the i-th, (i + nv)-th, ... block of
+// every warp.
 template <int KIND, int NB>
-__device__ __forceinline__ double sum_of(const RedItem &it, const int32_t *nb, int64_t b0,
-                                         int64_t b1)
+__device__ __forceinline__ void sums_of(const RedArgs &a, const RedItem &it, int64_t b0, int64_t b1,
+                                        double (&s)[4])
 {
-    if constexpr (NB != 0) return sum_uniform<KIND, NB>(it, b0, b1);
-    else return sum_mixed<KIND>(it, nb, b0, b1);
+    if constexpr (NB == 0) {
+        s[0] = sum_mixed<KIND>(it, a.nb, b0, b1);
+    } else {
+        if (a.nv == 4)
+            sum_uniform<KIND, NB, 4>(it, b0, b1, s);
+        else
+            sum_uniform<KIND, NB, 1>(it, b0, b1, s);
+    }
 }
 
 // Quantity blockIdx.z of cell blockIdx.y, NB orbitals per atom (0: any).
 template <int NB>
-__global__ void __launch_bounds__(RED_T, 3) k_reduce(const __grid_constant__ RedArgs a)
+__global__ void __launch_bounds__(RED_T, NB == 9 ? 3 : 4) k_reduce(const __grid_constant__ RedArgs a)
 {
+    __shared__ double sh[4][RED_T / 32];
     const RedItem &it = a.it[blockIdx.z];
     const int64_t unit = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
     const int64_t b0 = it.seg ? it.seg[blockIdx.y] : 0;
     const int64_t b1 = it.seg ? it.seg[blockIdx.y + 1] : it.nblk;
-    double s;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
     if (it.kind == RED_TRACE)
-        s = sum_of<RED_TRACE, NB>(it, a.nb, b0, b1);
+        sums_of<RED_TRACE, NB>(a, it, b0, b1, s);
     else if (it.kind == RED_DOT)
-        s = sum_of<RED_DOT, NB>(it, a.nb, b0, b1);
+        sums_of<RED_DOT, NB>(a, it, b0, b1, s);
     else
-        s = sum_of<RED_FROB_MI, NB>(it, a.nb, b0, b1);
-    s = cta_reduce<SUM>(s);
-    double *part = a.sink.part + unit * gridDim.x;
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+        sums_of<RED_FROB_MI, NB>(a, it, b0, b1, s);
+    // the tree of cta_reduce for the nv sums side by side (16 lanes hold nothing for 4 orbitals)
+#pragma unroll
+    for (int o = NB == 4 ? 8 : 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < a.nv) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sh[i][warp] = s[i];
+    __syncthreads();
+    double *part = a.sink.part + unit * (gridDim.x * a.nv);
+    if (warp < a.nv) {
+        double v = lane < RED_T / 32 ? sh[warp][lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            part[blockIdx.x + gridDim.x * warp] = v;
+            __threadfence();
+        }
+    }
     if (!last_arrival(a.sink, unit)) return;
-    s = fold<SUM>(part, 1);
+    const double v = fold<SUM>(part, gridDim.x * a.nv, 1);
     if (threadIdx.x == 0) {
-        a.sink.out[unit] = s;
+        a.sink.out[unit] = v;
         if (unit == 0) publish_flag(a.sink);
     }
 }
@@ -319,11 +346,12 @@ k_row_bounds(int n_atoms, const int32_t *cell_start, const int64_t *rp, const in
         part[3 * blockIdx.x + 0] = lo;
         part[3 * blockIdx.x + 1] = hi;
         part[3 * blockIdx.x + 2] = amax;
+        __threadfence();
     }
     if (!last_arrival(sink, blockIdx.y)) return;
-    lo = fold<MIN>(part + 0, 3);
-    hi = fold<MAX>(part + 1, 3);
-    amax = fold<MAX>(part + 2, 3);
+    lo = fold<MIN>(part + 0, gridDim.x, 3);
+    hi = fold<MAX>(part + 1, gridDim.x, 3);
+    amax = fold<MAX>(part + 2, gridDim.x, 3);
     if (threadIdx.x == 0) {
         double *o = sink.out + 3 * blockIdx.y;
         o[0] = lo;
@@ -453,7 +481,7 @@ __global__ void k_identity_seg(int n_atoms, const int32_t *cell_of, const int64_
 // CTAs of a unit with `work` CTAs' worth of items.
 cq_status red_sink(cq_ctx *ctx, int cells, int64_t work, int slot, RedSink *k, unsigned *ctas)
 {
-    const int64_t cap = std::max(RED_CELL, RED_G / cells);
+    const int64_t cap = cells == 1 ? RED_G : RED_CELL;
     void *p;
     cq_status st = cq_scratch(ctx, "red_part", sizeof(double) * RED_Q * cap * cells, &p);
     k->part = (double *)p;
@@ -493,9 +521,12 @@ cq_status cq_reduce(cq_ctx *ctx, int nq, const RedQ *q, bool per_cell, int slot)
     }
     a.nb = q[0].pA->geo->nb.as<int32_t>();
     unsigned ctas;
-    // a CTA takes 32 blocks (64 of 4 orbitals) at a time
-    cq_status st = red_sink(ctx, nc, (nblk / nc + 31) / 32, slot, &a.sink, &ctas);
+    cq_status st = red_sink(ctx, nc, nc > 1 ? RED_CELL : (nblk + 7) / 8, slot, &a.sink, &ctas);
     if (st != CQ_OK) return st;
+    // one cell of a uniform basis: four partials per CTA, so that all CTAs (256 at most) are
+    // resident and a warp has four blocks in flight even if it has no more than four
+    a.nv = nc > 1 || nbu == 0 ? 1 : 4;
+    ctas = (ctas + a.nv - 1) / a.nv;
     const dim3 grid(ctas, (unsigned)nc, (unsigned)nq);
     if (nbu == 9)
         k_reduce<9><<<grid, RED_T, 0, ctx->stream>>>(a);
