@@ -51,8 +51,9 @@ constexpr int E_MMAS = EMU_P * (EMU_P + 1) / 2;  // 36 plane products per K step
 
 struct EBars {
     uint64_t full[NSE], empty[NSE], acc_full, acc_empty, done;
-    uint64_t tile_full[NTQ], tile_empty[NTQ];
-    TileRec rec[NTQ];
+    static constexpr int TQ = 2;  // tiles queued ahead
+    uint64_t tile_full[TQ], tile_empty[TQ];
+    TileRec rec[TQ];
     uint32_t tmem_slot;
     int abort_flag;
 };
@@ -248,6 +249,40 @@ __device__ __forceinline__ void emu_produce(const EmuArgs &p, uint32_t sm0, EBar
     __syncwarp();
 }
 
+// The scheduler warp: hands out the launch's tiles in order, so that the tiles in flight on the
+// GPU stay neighbours (they share the A pieces of one or two M groups) and no CTA idles while
+// others hold several tiles.
+__device__ __forceinline__ void schedule(const EmuArgs &p, EBars *bars, volatile int *abort_flag,
+                                         int lane)
+{
+    if (lane == 0) {
+        int i = blockIdx.x;
+        for (uint32_t n = 0;; ++n) {
+            TileRec r;
+            r.tile = -1;
+            r.s0 = 0;
+            r.nks = r.nm = 0;
+            if (i < p.n_tiles) {
+                r.tile = i;
+                r.s0 = p.kstart[i];
+                r.nks = (int)(p.kstart[i + 1] - r.s0);
+                r.nm = 0;
+            }
+            if (n >= (uint32_t)EBars::TQ &&
+                !bar_wait(smem_u32(&bars->tile_empty[n % EBars::TQ]), ((n / EBars::TQ) + 1) & 1u, abort_flag))
+                break;
+            bars->rec[n % EBars::TQ] = r;
+            bar_arrive(smem_u32(&bars->tile_full[n % EBars::TQ]));
+            if (r.tile < 0) break;
+            i = (int)gridDim.x + (int)atomicAdd(&p.counter[0], 1u);
+        }
+        // the last CTA to finish handing out resets the counters for the next launch
+        __threadfence();
+        if (atomicInc(&p.counter[1], gridDim.x - 1) == gridDim.x - 1) atomicExch(&p.counter[0], 0u);
+    }
+    __syncwarp();
+}
+
 template <int NB>
 __global__ void __launch_bounds__(E_ST, 1) k_bsmm_emu(const EmuArgs p)
 {
@@ -268,7 +303,7 @@ __global__ void __launch_bounds__(E_ST, 1) k_bsmm_emu(const EmuArgs p)
         }
         init(&bars->acc_full, 1);
         init(&bars->acc_empty, 32 * E_DRAIN);
-        for (int r = 0; r < NTQ; ++r) {
+        for (int r = 0; r < EBars::TQ; ++r) {
             init(&bars->tile_full[r], 1);
             init(&bars->tile_empty[r], E_READERS);
         }
@@ -344,7 +379,7 @@ __global__ void __launch_bounds__(E_ST, 1) k_bsmm_emu(const EmuArgs p)
         }
         __syncwarp();
     } else if (warp == EW_SCHED) {
-        schedule(p, bars, abort_flag, lane, [](int) { return 0; });
+        schedule(p, bars, abort_flag, lane);
     } else {
         // ------------------------------------------------------------ drain and epilogue
         // at every tail step the warp drains the levels with the scales of the step's tail

@@ -60,7 +60,7 @@ constexpr int B_CHUNK = 3 * NT * KCH * 2;   // 18 KB
 constexpr int STAGE = A_CHUNK + B_CHUNK;    // one shared-memory stage of the split kernel
 constexpr int BAR_BYTES = 512;
 constexpr int DRAIN = 4;                     // chunks per FP32 accumulation period
-constexpr int NACC = 4;                      // FP32 accumulators in tensor memory
+constexpr int NACC = 8;                      // FP32 accumulators in tensor memory
 constexpr int TMEM_COLS = NACC * NT;
 constexpr long long WAIT_CYCLES = 4000000000LL;  // ~2 s at 2 GHz
 constexpr size_t A_PIECE_CAP = (size_t)12 << 30;  // scratch bound for one batch of A pieces

@@ -7,43 +7,53 @@
 //   warps 8, 9  producers of the A and of the B pieces: a chunk is up to three consecutive K
 //               steps of a tile; its pieces (main step: two A and two B main pieces; tail step:
 //               one A and one B tail piece; 18 KB either way) go into the step's slot of a
-//               free stage with TMA bulk copies that complete on the stage's "full" barrier;
-//   warp 10     one elected lane issues the MMAs of a chunk (6 split products per K step)
-//               into one of NACC TMEM accumulators (one per drain period, in rotation) and
-//               commits them to the stage's "empty" barrier, and at the end of a drain period
-//               to the accumulator's "full" barrier;
-//   warp 11     scheduler: takes the launch's next tile from a global counter and queues it for
-//               the other warps (NTQ tiles ahead).
-// Stages rotate over one running chunk counter across all tiles of the CTA; accumulators
-// over one running period counter; every wait computes its parity from those counters.
+//               free stage with TMA bulk copies that complete on the stage's "full" barrier.
+//               Lane 0 of warp 8 also takes the launch's tiles from a global counter and queues
+//               them for the other warps (TileFeed);
+//   warps 10, 11  MMA: each takes every second drain period; one elected lane issues the MMAs
+//               of a chunk (6 split products per K step) into one of NACC TMEM accumulators
+//               (one per drain period, in rotation) and commits them to the stage's "empty"
+//               barrier, and at the end of a drain period to the accumulator's "full" barrier.
+// The stages form one ring per MMA warp, each with a running chunk counter across all tiles of
+// the CTA (one warp alone waits on a stage, phase after phase); the chunks of two consecutive
+// periods of a tile are sent in turns.  Accumulators rotate over one running period counter;
+// every wait computes its parity from those counters.
 //
 // What bounds it, on the 4096-atom SZP cell's U.X kept on P_L (25.7 M K steps of 169 K per
-// SM, 18 KB each): first the issue of copies and MMAs from single-lane branches, then HBM.
-//  * A bulk copy costs its issuing thread 70-126 clocks whatever its size (one warp: 1291
-//    clocks for the 12 copies of a chunk; two warps work side by side), so two producer
-//    warps share a chunk, and pieces that are neighbours in memory move in one copy.
+// SM, 18 KB each): the issue of copies and MMAs, then shared memory (the operands of an MMA
+// of N = 64 take 48 clocks at 128 B per clock, a K step 150 ns).
+//  * A bulk copy costs its issuing thread 70-126 clocks whatever its size when its operands sit
+//    in per-lane registers, much less when they are warp-uniform (entries and tile records
+//    broadcast by shuffles, one elected lane).  Two producer warps share a chunk, and the two
+//    pieces of a step that are neighbours in memory move in one copy.  Chunks of one or two K
+//    steps cost more waits and barriers than they save (307 and 185 ns per step against 181).
 //  * tcgen05.mma (N = 64) issues at 68 clocks from a single-lane branch with descriptors in
-//    ordinary registers, at 58 from warp-uniform code with an elected lane; the operands
-//    alone take 48 (6 KB of shared memory at 128 B per clock).
+//    ordinary registers, at 58 from warp-uniform code with an elected lane, and a chunk's
+//    waits and commits add 140 during which nothing is issued: two warps on different
+//    accumulators cover each other.
 //  * With tiles dealt round-robin the CTAs drifted apart until the tiles in flight spanned
 //    ten M groups: 345 GB of DRAM reads, 7.2 TB/s.  The queue keeps them neighbours, and the
 //    B pieces (read once per tile) are evicted first, so the A pieces of one or two M groups
-//    (9 MB each) stay in L2.
-// Measured on that product: 316 ns per K step and SM before (53.5 ms with two producers in
-// place of one, 60.8 ms as it was), 282 with warp-uniform issue, 253 with the eviction
-// policies, 204 with the queue (34.6 ms).  The MMAs' own limit is 178 ns.
+//    (9 MB each) stay in L2.  Pairing periods across tiles, which needs tiles taken further
+//    ahead, cost more than it gave (L.S on 1728 atoms: 343 ns per step against 289).
+// Measured on that product, ns per K step and SM: 316 with two producers (360 with one), 282
+// with warp-uniform MMA issue, 253 with the eviction policies, 204 with the queue, 188 with two
+// MMA warps, 181 with warp-uniform copies (30.5 ms; 60.8 at first).  S.X on 512 atoms 214 -> 201 by
+// the last two; L.S on 1728 atoms, 36 steps a tile, 272 -> 289 (its odd third period is alone).
 //
 // Every wait is bounded (about two seconds) and also ends when another role has given up:
 // the CTA then stops issuing work, retires its own copies and MMAs (bounded), frees its
 // tensor memory and returns with bit 16 of the context flag set.
-constexpr int NS = 4;                  // shared-memory stages
+constexpr int NS = 4;                  // shared-memory stages, NR of each MMA warp
 constexpr int N_DRAIN = 256;           // drain threads
 constexpr int NPROD = 2;               // producer warps
-constexpr int W_PROD = 8, W_MMA = W_PROD + NPROD;  // first producer warp, MMA warp (0-7 drain)
-constexpr int W_SCHED = W_MMA + 1;     // scheduler warp
-constexpr int ST = 32 * (W_SCHED + 1); // threads per CTA (12 warps)
-constexpr int NTQ = 2;                 // tiles queued ahead
-constexpr int TILE_READERS = NPROD + 1 + N_DRAIN / 32;  // warps that read each queued tile
+constexpr int NMMA = 2;                // MMA warps
+constexpr int W_PROD = 8, W_MMA = W_PROD + NPROD;  // first producer and MMA warp (0-7 drain)
+constexpr int ST = 32 * (W_MMA + NMMA);            // threads per CTA (12 warps)
+constexpr int NTQ = 4;                 // slots of the tile queue
+constexpr int TILE_READERS = NPROD + NMMA + N_DRAIN / 32;  // warps that read each queued tile
+constexpr int PERIOD = KSTEPS * DRAIN; // K steps of a drain period
+constexpr int NR = NS / NMMA;
 
 // A queued tile: its index, first K step, K steps and main K steps (tile < 0: no more tiles)
 struct TileRec {
@@ -52,9 +62,10 @@ struct TileRec {
 };
 
 struct Bars {
-    uint64_t full[NS], empty[NS], acc_full[NACC], acc_empty[NACC], done;
-    uint64_t tile_full[NTQ], tile_empty[NTQ];
-    TileRec rec[NTQ];
+    uint64_t full[NS], empty[NS], acc_full[NACC], acc_empty[NACC], done[NMMA];
+    static constexpr int TQ = NTQ;
+    uint64_t tile_full[TQ], tile_empty[TQ];
+    TileRec rec[TQ];
     uint64_t never;  // no thread ever arrives here: the test-only wait on it must run out
     uint32_t tmem_slot;
     int abort_flag;
@@ -118,10 +129,14 @@ __device__ __forceinline__ TileRec next_tile(B *bars, uint32_t n, volatile int *
     r.tile = -1;
     r.s0 = 0;
     r.nks = r.nm = 0;
-    if (warp_wait(smem_u32(&bars->tile_full[n % NTQ]), (n / NTQ) & 1u, abort_flag)) {
-        r = bars->rec[n % NTQ];
-        __syncwarp();
-        if (lane == 0) bar_arrive(smem_u32(&bars->tile_empty[n % NTQ]));
+    if (warp_wait(smem_u32(&bars->tile_full[n % B::TQ]), (n / B::TQ) & 1u, abort_flag)) {
+        // broadcast, so that what follows from it is warp-uniform
+        const TileRec q = bars->rec[n % B::TQ];
+        r.tile = __shfl_sync(0xffffffffu, q.tile, 0);
+        r.nks = __shfl_sync(0xffffffffu, q.nks, 0);
+        r.nm = __shfl_sync(0xffffffffu, q.nm, 0);
+        r.s0 = __shfl_sync(0xffffffffu, q.s0, 0);
+        if (lane == 0) bar_arrive(smem_u32(&bars->tile_empty[n % B::TQ]));
     }
     return r;
 }
@@ -294,6 +309,77 @@ __device__ __forceinline__ void mma_step(uint32_t acc_addr, uint32_t a, uint32_t
             "r"(a + pq[x][0] * PA), "r"(b + pq[x][1] * PB), "r"(IDESC), "r"(x == 0 ? acc : 1u), "r"(hi));
 }
 
+// The chunks of a pair of drain periods that starts at K step `base` of a tile of nks: n0 of the
+// first period, n1 of the second (0: none).  They go through the stages in turns -- chunk j of
+// the first, chunk j of the second -- as long as the second has any.
+struct PairChunks {
+    int n0, n1;
+    __device__ __forceinline__ PairChunks(int nks, int base)
+        : n0((min(PERIOD, nks - base) + KSTEPS - 1) / KSTEPS),
+          n1((max(0, min(PERIOD, nks - base - PERIOD)) + KSTEPS - 1) / KSTEPS)
+    {
+    }
+};
+
+// Hands out the launch's tiles in order from a global counter, so that the tiles in flight on the
+// GPU stay neighbours (they share the A pieces of one or two M groups) and no CTA idles while
+// others hold several tiles.  Lane 0 of the A producer runs it between tiles; a record is fetched
+// one tile before it is queued, so its latency is not seen.  Queueing record n + 1 waits until
+// all warps have read record n + 1 - NTQ, whose predecessors' chunks are all sent by then.
+struct TileFeed {
+    TileRec rec;   // the next record to queue
+    uint32_t n;    // records queued
+    bool open;
+
+    __device__ __forceinline__ void load(const SplitArgs &p, int i)
+    {
+        rec.tile = -1;
+        rec.s0 = 0;
+        rec.nks = rec.nm = 0;
+        if (i < p.n_tiles) {
+            rec.tile = i;
+            rec.s0 = p.kstart[i];
+            rec.nks = (int)(p.kstart[i + 1] - rec.s0);
+            rec.nm = p.nmain[i];
+        }
+    }
+    __device__ __forceinline__ int take(const SplitArgs &p)
+    {
+        return (int)gridDim.x + (int)atomicAdd(&p.counter[0], 1u);
+    }
+    // queues the CTA's first two records
+    __device__ __forceinline__ void start(const SplitArgs &p, Bars *bars, volatile int *abort_flag)
+    {
+        n = 0;
+        open = true;
+        load(p, blockIdx.x);
+        post(p, bars, abort_flag);
+        post(p, bars, abort_flag);
+    }
+    // queues the next record and fetches the one after
+    __device__ __forceinline__ void post(const SplitArgs &p, Bars *bars, volatile int *abort_flag)
+    {
+        if (!open) return;
+        if (n >= (uint32_t)NTQ &&
+            !bar_wait(smem_u32(&bars->tile_empty[n % NTQ]), ((n / NTQ) + 1) & 1u, abort_flag)) {
+            open = false;
+            return;
+        }
+        bars->rec[n % NTQ] = rec;
+        bar_arrive(smem_u32(&bars->tile_full[n % NTQ]));
+        ++n;
+        open = rec.tile >= 0;
+        if (!open) return;
+        load(p, take(p));
+    }
+    // the last CTA to finish handing out resets the counters for the next launch
+    __device__ __forceinline__ void close(const SplitArgs &p)
+    {
+        __threadfence();
+        if (atomicInc(&p.counter[1], gridDim.x - 1) == gridDim.x - 1) atomicExch(&p.counter[0], 0u);
+    }
+};
+
 // One producer warp (SIDE 0: A pieces, 1: B pieces) over all chunks of the CTA's tiles.
 template <int SIDE>
 __device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *bars,
@@ -303,19 +389,25 @@ __device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *
     constexpr int SLOT = SIDE ? B_SLOT : A_SLOT;
     const uint8_t *mains = SIDE ? p.b_main : p.a_main - p.am0 * A_MAIN;
     const uint8_t *tails = SIDE ? p.b_tail : p.a_tail - p.at0 * A_TAIL;
-    const uint32_t dst0 = sm0 + (SIDE ? B_SLOTS : 0) + lane * SLOT;
+    const uint32_t dst0 = sm0 + (SIDE ? B_SLOTS : 0);
     static_assert(TAIL == 2 * MAIN, "a tail piece fills a step's slot like two main pieces");
-    // K steps come PB at a time, one per lane, loaded one batch ahead (the next tile's first
-    // batch during this tile's last)
-    constexpr int PB = 32 / KSTEPS * KSTEPS;
+    const bool el = elect_one();
+    // K steps come a pair of periods at a time, one per lane, loaded one pair ahead (the next
+    // tile's first pair during this tile's last)
+    constexpr int PB = 2 * PERIOD;
+    static_assert(PB <= 32, "a lane per K step of a pair of periods");
     auto load = [&](const TileRec &t, int base) {
         return lane < PB && base + lane < t.nks
                    ? __ldg(reinterpret_cast<const int2 *>(p.steps + t.s0 + base + lane) + SIDE)
                    : make_int2(0, 0);
     };
     const uint64_t policy = SIDE ? l2_evict_first() : l2_evict_last();
-    uint32_t cg = 0;  // running chunk counter
+    uint32_t cm[NMMA] = {0, 0};  // running chunk counters of the MMA warps
+    uint32_t pg0 = 0;            // running period counter
     bool ok = true;
+    TileFeed feed;
+    if (SIDE == 0 && lane == 0) feed.start(p, bars, abort_flag);
+    __syncwarp();
     TileRec t = next_tile(bars, 0, abort_flag, lane);
     int2 cur = load(t, 0);
     for (uint32_t n = 1; t.tile >= 0 && ok; ++n) {
@@ -326,34 +418,55 @@ __device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *
                 nxt = load(t, base + PB);
             } else {
                 tn = next_tile(bars, n, abort_flag, lane);
+                if (SIDE == 0 && lane == 0) feed.post(p, bars, abort_flag);
+                __syncwarp();
                 nxt = load(tn, 0);
             }
-            for (int q0 = base; q0 < min(t.nks, base + PB); q0 += KSTEPS, ++cg) {
-                const uint32_t s = cg % NS, fb = smem_u32(&bars->full[s]);
-                const int ex = __shfl_sync(0xffffffffu, cur.x, q0 - base + lane);
-                const int ey = __shfl_sync(0xffffffffu, cur.y, q0 - base + lane);
-                if (!warp_wait_lane0(cg >= (uint32_t)NS, smem_u32(&bars->empty[s]),
-                                     ((cg / NS) + 1) & 1u, abort_flag, lane)) {
+            const PairChunks pc(t.nks, base);
+            for (int c = 0; c < pc.n0 + pc.n1; ++c) {
+                // chunks in turns while the second period has any, then the first's rest
+                const int second = c < 2 * pc.n1 ? c & 1 : 0, j = c < 2 * pc.n1 ? c >> 1 : c - pc.n1;
+                const int q0 = base + second * PERIOD + j * KSTEPS;
+                const uint32_t m = (pg0 + second) & 1u, k = m ? cm[1] : cm[0];
+                const uint32_t s = NMMA * (k % NR) + m, fb = smem_u32(&bars->full[s]);
+                // broadcast entries, so that the copies' operands are warp-uniform
+                int ex[KSTEPS], ey[KSTEPS];
+#pragma unroll
+                for (int ks = 0; ks < KSTEPS; ++ks) {
+                    ex[ks] = __shfl_sync(0xffffffffu, cur.x, q0 - base + ks);
+                    ey[ks] = __shfl_sync(0xffffffffu, cur.y, q0 - base + ks);
+                }
+                if (k >= (uint32_t)NR &&
+                    !warp_wait(smem_u32(&bars->empty[s]), ((k / NR) + 1) & 1u, abort_flag)) {
                     ok = false;
                     break;
                 }
-                if (lane == 0)
+                const int nk = min(KSTEPS, t.nks - q0);
+                if (el) {
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
-                                 "r"((uint32_t)(min(KSTEPS, t.nks - q0) * SLOT))
+                                 "r"((uint32_t)(nk * SLOT))
                                  : "memory");
-                __syncwarp();
-                const int q = q0 + lane;
-                if (lane < KSTEPS && q < t.nks) {
-                    const uint32_t dst = dst0 + s * STAGE;
-                    const bool tail = q >= t.nm, pair = ey == ex + 1;
-                    bulk_copy(dst, tail ? tails + (int64_t)ex * TAIL : mains + (int64_t)ex * MAIN,
-                              tail || pair ? 2 * MAIN : MAIN, fb, policy);
-                    if (!tail && !pair)
-                        bulk_copy(dst + MAIN, ey < 0 ? p.zero : mains + (int64_t)ey * MAIN, MAIN, fb,
-                                  policy);
+#pragma unroll
+                    for (int ks = 0; ks < KSTEPS; ++ks) {
+                        if (ks >= nk) break;
+                        const uint32_t dst = dst0 + s * STAGE + ks * SLOT;
+                        if (q0 + ks >= t.nm) {
+                            bulk_copy(dst, tails + (int64_t)ex[ks] * TAIL, TAIL, fb, policy);
+                        } else if (ey[ks] == ex[ks] + 1) {
+                            bulk_copy(dst, mains + (int64_t)ex[ks] * MAIN, 2 * MAIN, fb, policy);
+                        } else {
+                            bulk_copy(dst, mains + (int64_t)ex[ks] * MAIN, MAIN, fb, policy);
+                            bulk_copy(dst + MAIN, ey[ks] < 0 ? p.zero : mains + (int64_t)ey[ks] * MAIN,
+                                      MAIN, fb, policy);
+                        }
+                    }
                 }
+                __syncwarp();
+                cm[0] += 1 - m;
+                cm[1] += m;
             }
             if (!ok) break;
+            pg0 += (pc.n0 > 0) + (pc.n1 > 0);  // (a tile without K steps has no period)
             cur = nxt;
         }
         t = tn;
@@ -362,45 +475,13 @@ __device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *
     // both sides: they arm the same chunks, since a free stage is seen by both (the barrier
     // is tried before the abort flag)
     if (lane == 0)
-        for (uint32_t k = 0; k < (uint32_t)NS && k < cg; ++k) {
-            const uint32_t c = cg - 1 - k;
-            if (!bar_wait_plain(smem_u32(&bars->full[c % NS]), (c / NS) & 1u)) *abort_flag = 1;
-        }
-    __syncwarp();
-}
-
-// The scheduler warp: hands out the launch's tiles in order, so that the tiles in flight on the
-// GPU stay neighbours (they share the A pieces of one or two M groups) and no CTA idles while
-// others hold several tiles.  nmain(tile): its main K steps.
-template <class Args, class B, class F>
-__device__ __forceinline__ void schedule(const Args &p, B *bars, volatile int *abort_flag, int lane,
-                                         F nmain)
-{
-    if (lane == 0) {
-        int i = blockIdx.x;
-        for (uint32_t n = 0;; ++n) {
-            TileRec r;
-            r.tile = -1;
-            r.s0 = 0;
-            r.nks = r.nm = 0;
-            if (i < p.n_tiles) {
-                r.tile = i;
-                r.s0 = p.kstart[i];
-                r.nks = (int)(p.kstart[i + 1] - r.s0);
-                r.nm = nmain(i);
+        for (uint32_t m = 0; m < NMMA; ++m)
+            for (uint32_t k = 0; k < (uint32_t)NR && k < cm[m]; ++k) {
+                const uint32_t c = cm[m] - 1 - k;
+                if (!bar_wait_plain(smem_u32(&bars->full[NMMA * (c % NR) + m]), (c / NR) & 1u))
+                    *abort_flag = 1;
             }
-            if (n >= (uint32_t)NTQ &&
-                !bar_wait(smem_u32(&bars->tile_empty[n % NTQ]), ((n / NTQ) + 1) & 1u, abort_flag))
-                break;
-            bars->rec[n % NTQ] = r;
-            bar_arrive(smem_u32(&bars->tile_full[n % NTQ]));
-            if (r.tile < 0) break;
-            i = (int)gridDim.x + (int)atomicAdd(&p.counter[0], 1u);
-        }
-        // the last CTA to finish handing out resets the counters for the next launch
-        __threadfence();
-        if (atomicInc(&p.counter[1], gridDim.x - 1) == gridDim.x - 1) atomicExch(&p.counter[0], 0u);
-    }
+    if (SIDE == 0 && lane == 0) feed.close(p);
     __syncwarp();
 }
 
@@ -436,7 +517,9 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->tile_empty[r])),
                          "r"(TILE_READERS));
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->done)), "r"(1));
+        for (int m = 0; m < NMMA; ++m)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->done[m])),
+                         "r"(1));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars->never)), "r"(1));
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -463,14 +546,15 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             produce<0>(p, sm0, bars, abort_flag, lane);
         else
             produce<1>(p, sm0, bars, abort_flag, lane);
-    } else if (warp == W_MMA) {
+    } else if (warp >= W_MMA) {
         // ------------------------------------------------------------ MMA issue
-        // the whole warp walks the chunks (uniform control flow keeps the descriptors in
-        // uniform registers: 58 clocks per MMA against 68 from a single-lane branch); one
-        // elected lane issues
+        // MMA warp m takes the periods of parity m.  The whole warp walks the
+        // chunks (uniform control flow keeps the descriptors in uniform registers: 58 clocks
+        // per MMA against 68 from a single-lane branch); one elected lane issues.
+        const int m = warp - W_MMA;
         const bool el = elect_one();
-        uint32_t cg = 0, pg = 0;
-        bool ok = true;
+        uint32_t cm = 0, pg0 = 0;  // chunks consumed, first period of the current pair
+        bool ok = true, issued = false;
         // test mode: the first wait is on a barrier nothing completes, with a short limit,
         // so it runs out; the CTA then takes the same abort path as a real timeout
         if (p.test_wait_cycles > 0) {
@@ -490,54 +574,57 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             const TileRec tr = next_tile(bars, n, abort_flag, lane);
             if (tr.tile < 0) break;
             const int nks = tr.nks, nm = tr.nm;
-            int period = 0;  // chunks of the current drain period already issued
-            for (int q0 = 0; q0 < nks; q0 += KSTEPS, ++cg) {
-                const uint32_t b = pg % NACC;
-                if (period == 0 && pg >= (uint32_t)NACC &&
-                    !warp_wait(bar0 + (uint32_t)offsetof(Bars, acc_empty) + 8 * b,
-                               ((pg / NACC) + 1) & 1u, abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t s = cg % NS;
-                if (!warp_wait(bar0 + (uint32_t)offsetof(Bars, full) + 8 * s, (cg / NS) & 1u,
-                               abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int base = 0; base < nks && ok; base += 2 * PERIOD) {
+                const PairChunks pc(nks, base);
+                const int second = (m ^ pg0) & 1, nc = second ? pc.n1 : pc.n0;
+                const uint32_t pg = pg0 + second, b = pg % NACC;
                 const uint32_t acc_addr = tmem + b * NT;
-                const bool last = q0 + KSTEPS >= nks || period == DRAIN - 1;
-                if (el) {
-#pragma unroll
-                    for (int ks = 0; ks < KSTEPS; ++ks) {
-                        if (q0 + ks >= nks) break;
-                        const uint32_t oa = s * (STAGE >> 4) + ks * (A_SLOT >> 4);
-                        const uint32_t ob = s * (STAGE >> 4) + ks * (B_SLOT >> 4);
-                        const uint32_t acc = period == 0 && ks == 0 ? 0u : 1u;
-                        // plane strides in 16-byte units: main pieces hold one column per
-                        // plane, tail pieces two
-                        if (q0 + ks < nm)
-                            mma_step<COLB_A / 16, COLB_B / 16>(acc_addr, dam + oa, dbm + ob, acc);
-                        else
-                            mma_step<2 * COLB_A / 16, 2 * COLB_B / 16>(acc_addr, dat + oa, dbt + ob, acc);
+                for (int j = 0; j < nc; ++j, ++cm) {
+                    if (j == 0 && pg >= (uint32_t)NACC &&
+                        !warp_wait(bar0 + (uint32_t)offsetof(Bars, acc_empty) + 8 * b,
+                                   ((pg / NACC) + 1) & 1u, abort_flag)) {
+                        ok = false;
+                        break;
                     }
-                    bar_commit(bar0 + (uint32_t)offsetof(Bars, empty) + 8 * s);
-                    if (last) bar_commit(bar0 + (uint32_t)offsetof(Bars, acc_full) + 8 * b);
+                    const uint32_t s = NMMA * (cm % NR) + m;
+                    const int q0 = base + second * PERIOD + j * KSTEPS;
+                    if (!warp_wait(bar0 + (uint32_t)offsetof(Bars, full) + 8 * s, (cm / NR) & 1u,
+                                   abort_flag)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (el) {
+#pragma unroll
+                        for (int ks = 0; ks < KSTEPS; ++ks) {
+                            if (q0 + ks >= nks) break;
+                            const uint32_t oa = s * (STAGE >> 4) + ks * (A_SLOT >> 4);
+                            const uint32_t ob = s * (STAGE >> 4) + ks * (B_SLOT >> 4);
+                            const uint32_t acc = j == 0 && ks == 0 ? 0u : 1u;
+                            // plane strides in 16-byte units: main pieces hold one column per
+                            // plane, tail pieces two
+                            if (q0 + ks < nm)
+                                mma_step<COLB_A / 16, COLB_B / 16>(acc_addr, dam + oa, dbm + ob, acc);
+                            else
+                                mma_step<2 * COLB_A / 16, 2 * COLB_B / 16>(acc_addr, dat + oa,
+                                                                           dbt + ob, acc);
+                        }
+                        bar_commit(bar0 + (uint32_t)offsetof(Bars, empty) + 8 * s);
+                        if (j == nc - 1)
+                            bar_commit(bar0 + (uint32_t)offsetof(Bars, acc_full) + 8 * b);
+                    }
+                    __syncwarp();
+                    issued = true;
                 }
-                __syncwarp();
-                period = last ? 0 : period + 1;
-                pg += last;
+                pg0 += pc.n1 ? 2 : 1;
             }
         }
         // retire every MMA before the tensor memory is released
-        if (cg > 0 && el) {
-            bar_commit(smem_u32(&bars->done));
-            if (!bar_wait_plain(smem_u32(&bars->done), 0u)) *abort_flag = 1;
+        if (issued && el) {
+            bar_commit(smem_u32(&bars->done[m]));
+            if (!bar_wait_plain(smem_u32(&bars->done[m]), 0u)) *abort_flag = 1;
         }
         __syncwarp();
-    } else if (warp == W_SCHED) {
-        schedule(p, bars, abort_flag, lane, [&](int tile) { return p.nmain[tile]; });
     } else {
         // ------------------------------------------------------------ drain and epilogue
         const int quarter = warp & 3, half = warp >> 2;
@@ -549,7 +636,7 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
             const TileRec tr = next_tile(bars, n, abort_flag, lane);
             if (tr.tile < 0) break;
             const int tile = tr.tile;
-            const int np = (tr.nks + KSTEPS * DRAIN - 1) / (KSTEPS * DRAIN);
+            const int np = (tr.nks + PERIOD - 1) / PERIOD;
             // this row's C blocks, loaded now and used after the tile's last period
             constexpr int NJ = epi_slots<NB, 32>();
             int32_t cid[NJ];

@@ -56,3 +56,22 @@ def test_packed_operands(n, rA, rB):
     err, _ = block_errors(oC, got, ref)
     assert np.all(err <= 67 * 2.0 ** -24 * scale + 1e-300)
     ctx.close()
+
+
+@pytest.mark.parametrize("rA,rB,rC", [(1.0, 1.0, 18.0), (6.0, 1.0, 25.0), (9.0, 9.0, 40.0)])
+def test_tiles_without_work(rA, rB, rC):
+    """C reaches farther than the operands: tiles with no K step at all between tiles with some."""
+    ctx = cq.Context(0)
+    cell = I.diamond_cell((6, 2, 2), a=10.26, sigma=0.2, seed=17, norb=9)
+    pA, pB, pC = (gpu_pattern(ctx, cell, x) for x in (rA, rB, rC))
+    a = I.random_blocks(cell, rA, 1, symmetric=False)
+    b = I.random_blocks(cell, rB, 2, symmetric=False)
+    C = ctx.empty(pC).fill_(7.0)
+    ctx.bsmm(1.0, pA, upload_pairs(ctx, pA, a), pB, upload_pairs(ctx, pB, b), 0.0, pC, C,
+             cq.CQ_SPLIT_BF16X3)
+    oA, oB, oC = (O.Pattern.of_cell(cell, x) for x in (rA, rB, rC))
+    vA, vB = O.scatter(oA, a), O.scatter(oB, b)
+    ref = O.bsmm(1.0, oA, vA, oB, vB, 0.0, oC)
+    err, _ = block_errors(oC, to_oracle(C, layout_index(pC, oC)), ref)
+    assert np.all(err <= 67 * 2.0 ** -24 * natural_scale(oA, vA, oB, vB, oC) + 1e-300)
+    ctx.close()
