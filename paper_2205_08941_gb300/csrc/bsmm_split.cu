@@ -30,8 +30,9 @@
 // 12 KB), and B pieces per N group likewise (64 rows: 3 KB and 6 KB).  Shared memory holds
 // a K step in an 18 KB slot, so every step costs the same; the descriptors of a main step
 // reach its second atom's column through the leading byte offset, those of a tail step
-// its second column.  The tile kernel moves each piece with one TMA bulk copy; one thread
-// issues the MMAs, eight warps drain the accumulators (bsmm_split_kernel.cuh).  A pieces
+// its second column.  The tile kernel moves a piece, or two that are neighbours in memory, with
+// one TMA bulk copy; two warps issue the MMAs, eight drain the accumulators
+// (bsmm_split_kernel.cuh).  A pieces
 // are packed in batches of M groups so that their scratch stays below A_PIECE_CAP bytes.
 //
 // Bases other than uniform 4 or 9 orbitals (mixed counts, batches of cells) use the same
@@ -657,7 +658,7 @@ __device__ __forceinline__ void emu_rows(const double *x, int n, int E, uint4 (&
 }
 
 // Emulated main pieces of entries [e0, e0 + n) (one thread per (entry, row)): as
-// k_pack_main, eight digit planes of orbitals 0-7 against the row's group exponent.
+// the main pieces of k_pack9, eight digit planes of orbitals 0-7 against the row's group exponent.
 template <int NB, bool LEFT>
 __global__ void __launch_bounds__(256)
 k_pack_main_emu(int64_t e0, int64_t n, const int32_t *index, const int32_t *main_tail,
