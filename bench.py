@@ -45,7 +45,7 @@ BF16_FALLBACK_TFLOPS = 1900.0
 FP64_TRAFFIC_PER_LAUNCH = 90.66e9
 # The same for the split-BF16 and the emulated-FP64 tile kernels (one ncu pass over one LNV
 # step of each leg; profiles/bsmm_split_ncu_si1728.md, profiles/bsmm_emu_ncu_si1728.md)
-SPLIT_TRAFFIC_PER_LAUNCH = 157.85e9
+SPLIT_TRAFFIC_PER_LAUNCH = 92.44e9
 EMU_TRAFFIC_PER_LAUNCH = 374.46e9
 TRAFFIC_SOURCE = "ncu dram bytes per launch, one LNV step of this cell"
 
