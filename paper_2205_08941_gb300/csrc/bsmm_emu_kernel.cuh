@@ -428,11 +428,13 @@ __global__ void __launch_bounds__(E_ST, 1) k_bsmm_emu(const EmuArgs p)
                     // scales first, so their loads overlap the wait for the accumulators: this
                     // row's 2^(E_A - 14), and in lane x column x's 2^E_B.  Groups without a
                     // nonzero value have zero sums and a poisoned group's are NaN: any scale
-                    // will do.  Exponents beyond 60 take the general path.
+                    // will do.  2^ea 2^eb has to be finite (0 x infinity would be NaN), so at most
+                    // 2^127: E_A from -60 to 81 and E_B from -60 to 60 take the single factor,
+                    // anything beyond the general path.
                     auto plain = [](int e) { return (e ^ (e >> 31)) == EMU_POISON ? 0 : e; };
                     const int ea = plain(p.scale_a[(int64_t)ea_ent * MT + arow]) - 14;
                     const int eb = plain(p.scale_b[(int64_t)eb_ent * NT + c0 + (lane % E_W)]);
-                    const bool fast = __all_sync(0xffffffffu, abs(ea) <= 74 && abs(eb) <= 60);
+                    const bool fast = __all_sync(0xffffffffu, ea >= -74 && ea <= 67 && abs(eb) <= 60);
                     const float fa = __uint_as_float((uint32_t)(ea + 127) << 23);
                     const float fb = __uint_as_float((uint32_t)(eb + 127) << 23);
                     if (!warp_wait(smem_u32(&bars->acc_full), pg & 1u, abort_flag)) {
