@@ -133,6 +133,17 @@ void cq_timing_end(cq_ctx *ctx);
 cq_status cq_fail(cq_ctx *ctx, cq_status st, const std::string &msg);
 cq_status cq_check_cuda(cq_ctx *ctx, cudaError_t e, const char *what);
 cq_status cq_alloc(cq_ctx *ctx, DevBuf &buf, size_t bytes);
+// Makes room for `rows` rows by alloc() if there is room for fewer; `have` is what there is room
+// for.  It is 0 from the moment alloc is called until it has succeeded: cq_alloc gives the old
+// memory up before it can be refused.
+template <class F> cq_status cq_grow_rows(int64_t &have, int64_t rows, F alloc)
+{
+    if (have >= rows) return CQ_OK;
+    have = 0;
+    const cq_status st = alloc();
+    if (st == CQ_OK) have = rows;
+    return st;
+}
 // Scratch buffer by name, grown (never shrunk) to at least `bytes`.
 cq_status cq_scratch(cq_ctx *ctx, const std::string &name, size_t bytes, void **out);
 // Exclusive scan of int64 counts (n entries) into out (n + 1 entries), out[n] = total.

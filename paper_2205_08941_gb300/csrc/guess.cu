@@ -954,15 +954,14 @@ namespace {
 
 cq_status ensure_act(cq_guess *g, int64_t rows)
 {
-    if (g->act_rows >= rows) return CQ_OK;
     int64_t per = 0;
     for (int l = 1; l <= g->n_layers; ++l) per += 2 * g->dims[l];
     per += g->dims[g->n_layers];  // dY
     per += 256;                   // dH scratch of the widest layer
     per += 256;
-    CQ_TRY(cq_alloc(g->ctx, g->act, sizeof(float) * per * rows));
-    g->act_rows = rows;
-    return CQ_OK;
+    return cq_grow_rows(g->act_rows, rows, [&] {
+        return cq_alloc(g->ctx, g->act, sizeof(float) * per * rows);
+    });
 }
 
 int64_t pad16(int64_t x) { return (x + 15) & ~(int64_t)15; }
@@ -983,20 +982,20 @@ struct TrainBufs {
 
 cq_status tc_rows(cq_guess *g, int64_t rows, bool train)
 {
-    if (g->hb_rows < rows) {
-        CQ_TRY(cq_alloc(g->ctx, g->hb, sizeof(__nv_bfloat16) * (size_t)(rows * (NDESC + 3 * NHID))));
-        g->hb_rows = rows;
-    }
-    if (!train || g->tr_rows >= rows) return CQ_OK;
-    const int64_t ld = pad16(rows);
-    const size_t f32 = sizeof(float) * (size_t)(ld * (6 * NHID + 2 * NOUT_PAD));
-    const size_t b16 = sizeof(__nv_bfloat16) *
-                       (size_t)(ld * ((NDESC + 3 * NHID) + (3 * NHID + NOUT_PAD) + (2 * NHID + NOUT_PAD)));
-    CQ_TRY(cq_alloc(g->ctx, g->tr, f32 + b16));
-    g->tr_rows = rows;
-    // the padding columns of the output layer's dZ rows stay zero
-    return cq_check_cuda(g->ctx, cudaMemsetAsync(g->tr.ptr, 0, f32 + b16, g->ctx->stream),
-                         "training buffers");
+    CQ_TRY(cq_grow_rows(g->hb_rows, rows, [&] {
+        return cq_alloc(g->ctx, g->hb, sizeof(__nv_bfloat16) * (size_t)(rows * (NDESC + 3 * NHID)));
+    }));
+    if (!train) return CQ_OK;
+    return cq_grow_rows(g->tr_rows, rows, [&] {
+        const int64_t ld = pad16(rows);
+        const size_t f32 = sizeof(float) * (size_t)(ld * (6 * NHID + 2 * NOUT_PAD));
+        const size_t b16 = sizeof(__nv_bfloat16) * (size_t)(ld * ((NDESC + 3 * NHID) + (3 * NHID + NOUT_PAD) +
+                                                                  (2 * NHID + NOUT_PAD)));
+        CQ_TRY(cq_alloc(g->ctx, g->tr, f32 + b16));
+        // the padding columns of the output layer's dZ rows stay zero
+        return cq_check_cuda(g->ctx, cudaMemsetAsync(g->tr.ptr, 0, f32 + b16, g->ctx->stream),
+                             "training buffers");
+    });
 }
 
 TrainBufs tc_train_bufs(cq_guess *g)
@@ -1086,10 +1085,8 @@ cq_status mlp_forward(cq_guess *g, const float *X, int64_t rows, std::vector<flo
 {
     cq_ctx *ctx = g->ctx;
     CQ_TRY(ensure_act(g, rows));
-    if (g->xin_rows < rows) {
-        CQ_TRY(cq_alloc(ctx, g->xin, sizeof(float) * NDESC * rows));
-        g->xin_rows = rows;
-    }
+    CQ_TRY(cq_grow_rows(g->xin_rows, rows,
+                        [&] { return cq_alloc(ctx, g->xin, sizeof(float) * NDESC * rows); }));
     k_norm_in<<<blocks_for(rows * NDESC), 256, 0, ctx->stream>>>(
         rows * NDESC, X, g->in_mean.as<float>(), g->in_scale.as<float>(), g->xin.as<float>());
     cq_count_launch();
