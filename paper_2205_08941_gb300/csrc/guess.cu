@@ -160,6 +160,7 @@ struct RowAtoms {
 };
 
 constexpr int DESC_T = 256, DESC_PAIRS = 64;  // threads and pairs at a time of k_descriptors
+constexpr int DESC_SMEM = 96 * 1024;  // its shared memory at most (two CTAs per SM)
 
 struct DescShared {
     double e1[DESC_PAIRS][3], e2[DESC_PAIRS][3], e3[DESC_PAIRS][3], m[DESC_PAIRS][3];
@@ -1255,14 +1256,16 @@ extern "C" cq_status cq_guess_descriptors(cq_ctx *ctx, const cq_pattern *pL, flo
     if (n == 0) return CQ_OK;
     Box3 box;
     for (int c = 0; c < 3; ++c) box.v[c] = pL->geo->box[c];
-    // a row's displacements and atoms are cached in shared memory while they fit 96 KB (two
-    // CTAs per SM): 1500 atoms; the rows of the method's P_L hold about 130
+    // a row's displacements and atoms are cached in shared memory while they fit DESC_SMEM: about
+    // 1800 atoms; the rows of the method's P_L hold about 130.  The kernel's limit is that of the
+    // longest row whatever this row needs: it belongs to the process, and another thread's call
+    // may come between setting it and the launch.
     const size_t cache = (size_t)pL->max_row * (3 * sizeof(double) + 3 * sizeof(float) + sizeof(int32_t));
-    const bool cached = sizeof(DescShared) + cache <= 96 * 1024;
+    const bool cached = sizeof(DescShared) + cache <= DESC_SMEM;
     auto k = cached ? k_descriptors<true> : k_descriptors<false>;
     const size_t smem = sizeof(DescShared) + (cached ? cache : 0);
     CQ_TRY(cq_check_cuda(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem), "descriptors"));
+                                                   DESC_SMEM), "descriptors"));
     k<<<pL->geo->n_atoms, DESC_T, smem, ctx->stream>>>(pair0, pairs, pL->col.as<int32_t>(),
                                                        pL->row_ptr.as<int64_t>(),
                                                        pL->geo->pos.as<double>(), box, desc, frames);
