@@ -333,7 +333,8 @@ k_descriptors(const int64_t *pair0, const int32_t *pairs, const int32_t *col, co
                                return x * x + y * y + z * z < R_ENV2_F && e != je && row.cols[e] != i;
                            },
                            look);
-            if (!__any_sync(0xffffffffu, eb >= 0))  // none so near: look at all of them
+            // none within R_ENV for certain (the FP32 filter decides beyond it): look at all of them
+            if (!__any_sync(0xffffffffu, eb >= 0 && best <= R_ENV * R_ENV))
                 for (int base = 0; base < row.n; base += 32) {
                     const int e = base + lane;
                     look(e < row.n && e != je && row.cols[e] != i ? e : -1);
