@@ -523,9 +523,10 @@ cq_status cq_reduce(cq_ctx *ctx, int nq, const RedQ *q, bool per_cell, int slot)
     unsigned ctas;
     cq_status st = red_sink(ctx, nc, nc > 1 ? RED_CELL : (nblk + 7) / 8, slot, &a.sink, &ctas);
     if (st != CQ_OK) return st;
-    // one cell of a uniform basis: four partials per CTA, so that all CTAs (256 at most) are
-    // resident and a warp has four blocks in flight even if it has no more than four
-    a.nv = nc > 1 || nbu == 0 ? 1 : 4;
+    // one cell on a kernel of its basis: four partials per CTA, so that all CTAs (256 at most) are
+    // resident and a warp has four blocks in flight even if it has no more than four; the kernel
+    // for any basis makes one
+    a.nv = nc == 1 && (nbu == 9 || nbu == 4) ? 4 : 1;
     ctas = (ctas + a.nv - 1) / a.nv;
     const dim3 grid(ctas, (unsigned)nc, (unsigned)nq);
     if (nbu == 9)
