@@ -1453,13 +1453,14 @@ extern "C" cq_status cq_guess_train_step(cq_guess *g, const float *desc, const f
                              "loss sums"));
     }
     AdamArgs up = {lr > 0.f ? lr : 0.f, 0.9f, 0.999f, 1e-8f, 1.f, 1.f};
+    const int64_t step = g->step + (lr > 0.f ? 1 : 0);  // (a step that is refused does not count)
     if (lr > 0.f) {
-        g->step += 1;
-        up.c1 = 1.f - std::pow(up.b1, (float)g->step);
-        up.c2 = 1.f - std::pow(up.b2, (float)g->step);
+        up.c1 = 1.f - std::pow(up.b1, (float)step);
+        up.c2 = 1.f - std::pow(up.b2, (float)step);
     }
     CQ_TRY((g->fp32_weights ? train_fp32 : train_tc)(g, desc, targets, rows, (float *)vloss,
                                                      g->loss_acc.as<double>(), up));
+    g->step = step;
     if (loss_host) {
         float part[256];
         cudaMemcpyAsync(part, vloss, sizeof(part), cudaMemcpyDeviceToHost, s);

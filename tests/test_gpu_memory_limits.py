@@ -48,3 +48,29 @@ def test_refused_growth_of_the_networks_buffers(fp32):
     assert g.train_step(X, T, 0.0) == loss
     g.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("fp32", [False, True])
+def test_refused_training_step_is_no_step(fp32):
+    """Adam's step count advances with the weights only."""
+    X, T = batch(300)
+
+    def train(refusals):
+        ctx = cq.Context(0)
+        g = cq.Guess(ctx, seed=3, fp32_weights=fp32)
+        for _ in range(3):
+            if refusals:
+                ctx.set_mem_limit(1)
+                Xl, Tl = batch(5000, seed=2)
+                with pytest.raises(cq.CQError) as e:
+                    g.train_step(Xl, Tl, 1e-3)
+                assert e.value.status == 3
+                ctx.set_mem_limit(0)
+            g.train_step(X, T, 1e-3)
+        w, b = g.params()
+        g.close()
+        ctx.close()
+        return w, b
+
+    for x, y in zip(train(True), train(False)):
+        assert np.array_equal(x, y)
