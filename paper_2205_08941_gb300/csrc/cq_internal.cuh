@@ -100,7 +100,9 @@ struct cq_ctx {
     int64_t mem_used = 0;
     uint64_t next_id = 1;
     int num_sms = 0;
-    DevBuf flag;                     // int32 device error word
+    // int32 device error word, the tile queue's two counters (zero between launches), and from
+    // byte 16 the double that the FP64 probe could write to
+    DevBuf flag;
     DevBuf red_count;                // uint32 arrivals of a reduction's CTAs (zero between launches)
     double *host_out = nullptr;      // pinned host scalars; the last one is the error word
     std::map<std::tuple<uint64_t, uint64_t, uint64_t>, std::unique_ptr<TaskList>> tasks;

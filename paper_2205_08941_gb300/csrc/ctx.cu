@@ -257,13 +257,13 @@ extern "C" cq_status cq_ctx_create(int device, void *cuda_stream, cq_ctx **out)
     ctx->device = device;
     ctx->stream = (cudaStream_t)cuda_stream;
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
-    if (cq_alloc(ctx, ctx->flag, 16) != CQ_OK ||
+    if (cq_alloc(ctx, ctx->flag, 24) != CQ_OK ||
         cq_alloc(ctx, ctx->red_count, CQ_RED_SLOTS * 4) != CQ_OK ||
         cudaMallocHost(&ctx->host_out, CQ_RED_SLOTS * sizeof(double)) != cudaSuccess) {
         delete ctx;
         return CQ_ERR_NOMEM;
     }
-    cudaMemsetAsync(ctx->flag.ptr, 0, 16, ctx->stream);
+    cudaMemsetAsync(ctx->flag.ptr, 0, 24, ctx->stream);
     cudaMemsetAsync(ctx->red_count.ptr, 0, CQ_RED_SLOTS * 4, ctx->stream);
     ctx->host_out[CQ_RED_SLOTS - 1] = 0.0;
     *out = ctx;
@@ -744,11 +744,9 @@ extern "C" cq_status cq_peak_fp64(cq_ctx *ctx, double *flops_per_s_host)
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
-    void *v;
-    cq_status st = cq_scratch(ctx, "peak_sink", sizeof(double), &v);
-    if (st != CQ_OK) return st;
-    double *sink = (double *)v;
+    double *sink = ctx->flag.as<double>() + 2;  // (the probe allocates nothing)
     double best = 0.0;
+    cq_status st = CQ_OK;
     for (int kind = 0; kind < 2 && st == CQ_OK; ++kind) {
         const int it = kind == 0 ? iters : iters / 4;
         auto launch = [&](double seed) {

@@ -74,3 +74,10 @@ def test_refused_training_step_is_no_step(fp32):
 
     for x, y in zip(train(True), train(False)):
         assert np.array_equal(x, y)
+
+
+def test_fp64_probe_needs_no_memory():
+    ctx = cq.Context(0)
+    ctx.set_mem_limit(max(1, ctx.mem_used()))
+    assert ctx.peak_fp64() > 1e11
+    ctx.close()
