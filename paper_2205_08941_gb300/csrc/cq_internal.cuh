@@ -111,6 +111,7 @@ struct cq_ctx {
     std::map<std::string, std::unique_ptr<DevBuf>> scratch;
     std::vector<cq_pattern *> live_patterns;
     std::vector<cq_lnv *> live_lnv;
+    std::vector<cq_guess *> live_guess;
     // other cached per-pattern data, keyed (kind, id, id, id); entries naming a destroyed
     // pattern's id are dropped with it
     std::map<std::tuple<int, uint64_t, uint64_t, uint64_t>, std::shared_ptr<void>> aux;
@@ -242,6 +243,7 @@ static inline int64_t cq_pad2(int64_t x) { return (x + 1) & ~int64_t(1); }
 
 // Called by cq_ctx_destroy for LNV objects still alive: they stop touching the context.
 void cq_lnv_detach(cq_lnv *s);
+void cq_guess_detach(cq_guess *g);
 // G_N = 12(U - R3) only (the electron-number gradient) on P_L.
 cq_status cq_lnv_gradient_n(cq_ctx *ctx, const cq_pattern *pL, const cq_pattern *pU,
                             const double *U, const double *R3, double *GN);

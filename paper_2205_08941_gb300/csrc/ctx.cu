@@ -280,6 +280,7 @@ extern "C" void cq_ctx_destroy(cq_ctx *ctx)
         cudaEventDestroy(e.second);
     }
     for (cq_lnv *s : ctx->live_lnv) cq_lnv_detach(s);
+    for (cq_guess *g : ctx->live_guess) cq_guess_detach(g);
     for (auto &kv : ctx->derived) delete kv.second;
     ctx->derived.clear();
     for (cq_pattern *p : ctx->live_patterns) {

@@ -15,6 +15,7 @@
 // 1.2, cosine cut at 8) and the 9 real harmonics Y_a up to l = 2.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <random>
 
@@ -1161,21 +1162,35 @@ extern "C" cq_status cq_guess_create(cq_ctx *ctx, uint64_t seed, int32_t fp32_we
     cudaMemsetAsync(g->w4.ptr, 0, sizeof(__nv_bfloat16) * NHID * NOUT_PAD, s);
     refresh_weights(g.get(), s);
     CQ_TRY(cq_check_cuda(ctx, cudaStreamSynchronize(s), "guess create"));
+    ctx->live_guess.push_back(g.get());
     *out = g.release();
     return CQ_OK;
+}
+
+void cq_guess_detach(cq_guess *g)
+{
+    g->ctx = nullptr;
+    for (DevBuf *b : {&g->w, &g->wb, &g->b, &g->gw, &g->gb, &g->mw, &g->vw, &g->mb, &g->vb, &g->mean,
+                      &g->scale, &g->in_mean, &g->in_scale, &g->xin, &g->act, &g->wt, &g->w4, &g->hb,
+                      &g->tr, &g->loss_acc})
+        b->ctx = nullptr;
 }
 
 extern "C" void cq_guess_destroy(cq_guess *g)
 {
     if (!g) return;
-    if (g->ctx) cudaStreamSynchronize(g->ctx->stream);
+    if (g->ctx) {
+        cudaStreamSynchronize(g->ctx->stream);
+        auto &v = g->ctx->live_guess;
+        v.erase(std::find(v.begin(), v.end(), g));
+    }
     delete g;
 }
 
 extern "C" cq_status cq_guess_params(cq_guess *g, float *w_host, float *b_host, int64_t *n_w,
                                      int64_t *n_b, int32_t set)
 {
-    if (!g) return CQ_ERR_INVALID;
+    if (!g || !g->ctx) return CQ_ERR_INVALID;
     if (n_w) *n_w = g->n_w;
     if (n_b) *n_b = g->n_b;
     cudaStream_t s = g->ctx->stream;
@@ -1193,7 +1208,7 @@ extern "C" cq_status cq_guess_params(cq_guess *g, float *w_host, float *b_host, 
 extern "C" cq_status cq_guess_fit_scale(cq_guess *g, const float *desc, const float *targets,
                                         int64_t rows)
 {
-    if (!g || !desc || !targets || rows <= 0) return CQ_ERR_INVALID;
+    if (!g || !g->ctx || !desc || !targets || rows <= 0) return CQ_ERR_INVALID;
     cudaStream_t s = g->ctx->stream;
     k_colstats<<<1, 128, 0, s>>>(rows, NDESC, desc, g->in_mean.as<float>(), g->in_scale.as<float>());
     k_colstats<<<1, 128, 0, s>>>(rows, NOUT, targets, g->mean.as<float>(), g->scale.as<float>());
@@ -1205,7 +1220,7 @@ extern "C" cq_status cq_guess_set_scale(cq_guess *g, const float *in_mean_host,
                                         const float *in_scale_host, const float *out_mean_host,
                                         const float *out_scale_host)
 {
-    if (!g || !in_mean_host || !in_scale_host || !out_mean_host || !out_scale_host)
+    if (!g || !g->ctx || !in_mean_host || !in_scale_host || !out_mean_host || !out_scale_host)
         return CQ_ERR_INVALID;
     cudaStream_t s = g->ctx->stream;
     cudaMemcpyAsync(g->in_mean.ptr, in_mean_host, 4 * NDESC, cudaMemcpyHostToDevice, s);
@@ -1294,7 +1309,7 @@ extern "C" cq_status cq_guess_targets(cq_ctx *ctx, const cq_pattern *pL, const d
 
 extern "C" cq_status cq_guess_forward(cq_guess *g, const float *desc, int64_t rows, float *out)
 {
-    if (!g || !desc || !out || rows < 0) return CQ_ERR_INVALID;
+    if (!g || !g->ctx || !desc || !out || rows < 0) return CQ_ERR_INVALID;
     if (rows == 0) return CQ_OK;
     if (!g->fp32_weights) {
         CQ_TRY(tc_rows(g, rows, false));
@@ -1442,7 +1457,7 @@ extern "C" cq_status cq_guess_train_step(cq_guess *g, const float *desc, const f
                                          int64_t rows, float lr, float *loss_host,
                                          float *grad_w_host, float *grad_b_host)
 {
-    if (!g || !desc || !targets || rows <= 0) return CQ_ERR_INVALID;
+    if (!g || !g->ctx || !desc || !targets || rows <= 0) return CQ_ERR_INVALID;
     cq_ctx *ctx = g->ctx;
     cudaStream_t s = ctx->stream;
     void *vloss;
@@ -1481,7 +1496,7 @@ extern "C" cq_status cq_guess_train_step(cq_guess *g, const float *desc, const f
 extern "C" cq_status cq_guess_loss_sum(cq_guess *g, double *sq_sum_host, int64_t *rows_host,
                                        int32_t reset)
 {
-    if (!g) return CQ_ERR_INVALID;
+    if (!g || !g->ctx) return CQ_ERR_INVALID;
     cq_ctx *ctx = g->ctx;
     double v[2] = {0.0, 0.0};
     if (g->loss_acc.ptr) {
@@ -1498,7 +1513,7 @@ extern "C" cq_status cq_guess_loss_sum(cq_guess *g, double *sq_sum_host, int64_t
 // frame; writes all (i, j) and (j, i) blocks of L.
 extern "C" cq_status cq_guess_apply(cq_guess *g, const cq_pattern *pL, double *L)
 {
-    if (!g || !pL || !L) return CQ_ERR_INVALID;
+    if (!g || !g->ctx || !pL || !L) return CQ_ERR_INVALID;
     cq_ctx *ctx = g->ctx;
     const int nb = pL->geo->uniform_nb;
     if (nb != 9 && nb != 4) return cq_fail(ctx, CQ_ERR_INVALID, "guess: uniform 4 or 9 orbitals");
