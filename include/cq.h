@@ -197,9 +197,10 @@ cq_status cq_pattern_scatter(cq_ctx *ctx, const cq_pattern *p, int64_t n_pairs,
  * of K in the spatial (Morton) order (four for a 4-orbital basis) a power-of-two scale 2^E
  * with |x| < 2^E; every value is rounded to the grid
  * 2^(E-63) and cut into eight signed 8-bit digits, each exact in BF16; the 36 digit
- * products of levels p + q <= 7 run on the tensor cores, levels 0-4 summed exactly in FP32
- * within a scale period and levels 5-7 together, and every period drains into a three-float
- * (about 72-bit) sum.  Every value is carried to 2^-64 of its group's largest magnitude,
+ * products of levels p + q <= 7 run on the tensor cores, every level in an FP32 accumulator of
+ * its own (exact for levels 0-6 within a scale period), and every period drains into a
+ * three-float (about 72-bit) sum: levels 0-4 without error, levels 5-7 rounded together at
+ * 2^-65 of the bound of level 0.  Every value is carried to 2^-64 of its group's largest magnitude,
  * so the error of C_ij stays below about 1e-15 sum_k (Amax ||B_kj|| + ||A_ik|| Bmax) with
  * Amax, Bmax the largest magnitudes of the scale groups the terms fall in.  While the
  * magnitudes inside a group stay within about 2^14 of one another (the smooth decay of the

@@ -13,9 +13,11 @@
 // steps pairing the tile's K atoms of the group, then the group's tail step.
 //
 // At a period's end the drain warps compress every element's eight level sums into three
-// floats (x0, x1, x2) without error down to about 2^-72 and add them, scaled by
-// 2^(E_A(row) + E_B(column) - 14), into a three-float sum (h, m, l) in registers: 45 FP32
-// operations per element (84 when each level was scaled and added by itself).
+// floats (x0, x1, x2) and add them, scaled by 2^(E_A(row) + E_B(column) - 14), into a
+// three-float sum (h, m, l) in registers: 45 FP32 operations per element (84 when each level was
+// scaled and added by itself).  Levels 0-4 are compressed without error; levels 5-7 are added in
+// FP32 first, which loses at most 2^-65 of level 0's bound (2^-65.0 in a CPU emulation of sums
+// spread over their whole ranges, 2^-68 with Gaussian ones): the digits resolve 2^-64.
 // After a tile's last period C = beta C + alpha (h + m + l) is written in FP64.
 //
 // Warp roles: as in the split kernel, with 16 drain warps (four to a scheduler, sixteen columns
@@ -130,13 +132,6 @@ __device__ __forceinline__ void emu_compress(const uint32_t (&v)[EMU_P], float &
 }
 
 constexpr int E_C = 4;  // columns drained together
-
-__device__ __forceinline__ void tm_ld(uint32_t addr, uint32_t (&v)[2])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];"
-                 : "=r"(v[0]), "=r"(v[1])
-                 : "r"(addr));
-}
 
 __device__ __forceinline__ void tm_ld(uint32_t addr, uint32_t (&v)[4])
 {

@@ -18,8 +18,9 @@ constexpr int F64_T = 64;
 
 // One or two products over the same task list (blockIdx.y picks the operands): the pairs of an
 // LNV evaluation that share their patterns go in one launch.  A 64-atom cell's product is one
-// wave of short dependent chains (22 us alone), so its partner runs beside it for little: an
-// LNV run at 64 atoms takes 6.3 ms (7.4 ms with one product per launch and 16 lanes per row).
+// wave of short dependent chains (18 us alone), so its partner runs beside it for little: pairs
+// and the lane split below took an LNV run at 64 atoms from 7.4 to 6.3 ms (it is 4.0 ms now, with
+// the one-launch reductions and the small CTAs).
 struct F64Ops {
     const double *A[2], *B[2];
     double *C[2];

@@ -472,7 +472,8 @@ k_pack9(int64_t t0, int64_t m0, const int32_t *t_group, const int32_t *t_key, co
 
 // Tail pieces of entries [e0, e0 + n) (one thread per (entry, row)), entry = (atom group,
 // tail group), index = its block per (slot, atom u of the tail group).  K position
-// u * TW + m (two core columns) = orbital MAINW + m of atom u.
+// u * TW + m (two core columns) = orbital MAINW + m of atom u.  4-orbital bases only, whose atoms
+// have no main pieces (k_pack9 makes the pieces of 9 orbitals).
 template <int NB, bool LEFT>
 __global__ void __launch_bounds__(256)
 k_pack_tail(int64_t e0, int64_t n, const int32_t *index, const double *__restrict__ X,
@@ -506,18 +507,6 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x)
     const float err = (hi - (s - bp)) + (x - bp);
     hi = s;
     lo += err;
-}
-
-// float -> double by its bits (a select for zeros, the conversion only for denormals,
-// infinities and NaNs): conversions to 64 bits run at the FP64 pipe's two lanes per clock and
-// SM, integer operations at 64 and more
-__device__ __forceinline__ double f32_to_f64(float x)
-{
-    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
-    if (m - 1u >= 0x007fffffu && m < 0x7f800000u)  // zero or normal
-        return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u)),
-                                (int)(u << 29));
-    return (double)x;
 }
 
 struct SplitArgs {

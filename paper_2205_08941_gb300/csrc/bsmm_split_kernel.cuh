@@ -471,9 +471,10 @@ __device__ __forceinline__ void produce(const SplitArgs &p, uint32_t sm0, Bars *
         }
         t = tn;
     }
-    // every copy lands before the CTA's shared memory is released.  A stage's barrier needs
-    // both sides: they arm the same chunks, since a free stage is seen by both (the barrier
-    // is tried before the abort flag)
+    // every copy lands before the CTA's shared memory is released.  A stage's barrier needs both
+    // sides.  They arm the same chunks unless the CTA is giving up: then one side may have found a
+    // stage busy and left, and the other finds it free and arms it.  Its wait below runs out after
+    // two seconds (the flag is set already), and its own copies have long landed by then.
     if (lane == 0)
         for (uint32_t m = 0; m < NMMA; ++m)
             for (uint32_t k = 0; k < (uint32_t)NR && k < cm[m]; ++k) {
@@ -538,10 +539,9 @@ __global__ void __launch_bounds__(ST, 1) k_bsmm_split(const SplitArgs p)
 
     if (warp == W_PROD || warp == W_PROD + 1) {
         // ------------------------------------------------------------ producers
-        // warp W_PROD copies the A pieces of every chunk, the next warp the B pieces; lane x
-        // those of the chunk's K step x.  The two main pieces of a step are neighbours in
-        // memory when no atom of the group's list lies between the two, and then one copy
-        // moves both.
+        // warp W_PROD copies the A pieces of every chunk, the next warp the B pieces (one elected
+        // lane issues them).  The two main pieces of a step are neighbours in memory when no atom
+        // of the group's list lies between the two, and then one copy moves both.
         if (warp == W_PROD)
             produce<0>(p, sm0, bars, abort_flag, lane);
         else

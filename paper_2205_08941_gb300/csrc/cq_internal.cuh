@@ -52,7 +52,8 @@ struct Geometry {
     DevBuf cell_of, boxes_dev, cell_start_dev;
 };
 
-// (i, k, j) task list of mask_{P_C}(A.B), sorted by C block then k ascending.
+// (i, k, j) task list of mask_{P_C}(A.B), sorted by C block, then (on a mixed basis) by the orbital
+// count of k, then k ascending.
 struct TaskList {
     int64_t n_c = 0;
     int64_t n_tasks = 0;
@@ -240,6 +241,18 @@ void cq_capture_counting(bool on);
 int64_t cq_capture_launches(void);
 
 static inline int64_t cq_pad2(int64_t x) { return (x + 1) & ~int64_t(1); }
+
+// float -> double by its bits (a select for zeros, the conversion only for denormals,
+// infinities and NaNs): conversions to 64 bits run at the FP64 pipe's two lanes per clock and
+// SM, integer operations at 64 and more
+__device__ __forceinline__ double f32_to_f64(float x)
+{
+    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m - 1u >= 0x007fffffu && m < 0x7f800000u)  // zero or normal
+        return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u)),
+                                (int)(u << 29));
+    return (double)x;
+}
 
 // Called by cq_ctx_destroy for LNV objects still alive: they stop touching the context.
 void cq_lnv_detach(cq_lnv *s);

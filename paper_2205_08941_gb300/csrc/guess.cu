@@ -454,17 +454,6 @@ __global__ void k_targets(int64_t n_pairs, int nb, int stride, const int32_t *pa
         }
 }
 
-// float -> double by its bits for zeros and normal numbers (conversions to 64 bits run at the
-// FP64 pipe's two lanes per clock and SM)
-__device__ __forceinline__ double f32_to_f64(float x)
-{
-    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
-    if (m - 1u >= 0x007fffffu && m < 0x7f800000u)
-        return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u)),
-                                (int)(u << 29));
-    return (double)x;
-}
-
 // The d-shell rotation D2[a][b] = <Q_b, R^T Q_a R>_F of frame rows R, with the forms' few
 // non-zero entries only (the terms and their order are orbital_rotation's)
 __device__ __forceinline__ void d_rotation(const double (&R)[3][3], double (*D2)[5])

@@ -12,7 +12,7 @@
 //
 // What bounds a training step of 4096 rows: launches and latency (a layer is 0.5 GFLOP and
 // 4 MB).  In 48 launches of separate passes, with column sums of one thread per column, it
-// took 806 us; in these 11 launches about 135 us.
+// took 806 us; in these 11 launches about 154 us.
 //
 // The MMA completion wait is bounded (about two seconds); a CTA that gives up sets bit 16
 // of the flag word, frees its tensor memory and returns.

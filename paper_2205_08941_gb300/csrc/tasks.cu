@@ -1,11 +1,11 @@
 // Device-built (i, k, j) task lists of the masked product mask_{P_C}(A.B), and block maps
 // between patterns.
 //
-// For C block (i, j) the tasks are every k with (i, k) in P_A and (k, j) in P_B (in
-// ascending k; on a mixed basis by the orbital count of k first).  Every pattern is symmetric, so (k, j) in P_B <=> k in row j of P_B: the
-// k set is the intersection of two sorted rows.  A task is stored as the pair
-// (index of block (i, k) in P_A, index of block (k, j) in P_B) -- the latter through P_B's
-// transpose map -- so the product kernels never search.
+// For C block (i, j) the tasks are every k with (i, k) in P_A and (k, j) in P_B (in ascending k;
+// on a mixed basis by the orbital count of k first).  Every pattern is symmetric, so
+// (k, j) in P_B <=> k in row j of P_B: the k set is the intersection of two sorted rows.  A
+// task is stored as the pair (index of block (i, k) in P_A, index of block (k, j) in P_B) --
+// the latter through P_B's transpose map -- so the product kernels never search.
 #include "cq_internal.cuh"
 
 namespace {
