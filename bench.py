@@ -39,15 +39,15 @@ WORKLOAD = {"workload": "Si diamond 4096 atoms SZP (9 orb/atom, 36864 orbitals)"
             "ncell": 8, "a_bohr": 10.26, "sigma_bohr": 0.1, "seed": 2, "r_S": 14.0,
             "r_L": 16.0, "r_X": 30.0, "r_U": 44.0, "n_electrons": 16384}
 BF16_FALLBACK_TFLOPS = 1900.0
-# DRAM bytes per launch of the FP64 product kernel over the launches of one LNV step of the
-# 4096-atom cell, from one ncu capture of the current kernel
-# (profiles/bsmm_f64_traffic_si4096.md)
-FP64_TRAFFIC_PER_LAUNCH = 90.66e9
-# The same for the split-BF16 and the emulated-FP64 tile kernels (one ncu pass over one LNV
-# step of each leg; profiles/bsmm_split_ncu_si1728.md, profiles/bsmm_emu_ncu_si1728.md)
+# DRAM bytes per launch of each leg's product kernel over the launches of the first timed LNV step
+# of the 4096-atom cell, from one-pass ncu captures (profiles/bsmm_f64_traffic_si4096.md,
+# profiles/bsmm_split_ncu_si1728.md, profiles/bsmm_emu_ncu_si1728.md).  An FP64 launch holds one
+# product or two (27 launches, 32 products: 90.8 GB per product); captured again whenever a
+# kernel, its launches or the plan changes.
+FP64_TRAFFIC_PER_LAUNCH = 107.66e9
 SPLIT_TRAFFIC_PER_LAUNCH = 92.44e9
-EMU_TRAFFIC_PER_LAUNCH = 374.46e9
-TRAFFIC_SOURCE = "ncu dram bytes per launch, one LNV step of this cell"
+EMU_TRAFFIC_PER_LAUNCH = 222.78e9
+TRAFFIC_SOURCE = "ncu dram bytes per launch, one LNV step of this cell (a capture, not this run)"
 
 
 METRIC = ("block-sparse GEMM GFLOP/s (useful FP64 flops) & s per LNV step, Si SZP; "
@@ -415,6 +415,16 @@ def make_inputs(ncell):
                           seed=WORKLOAD["seed"], norb=9)
     S, H = I.overlap_hamiltonian(cell, I.silicon_model(WORKLOAD["r_S"]))
     return cell, S, H
+
+
+def fp64_peak(probe, n_sms, sm_max_mhz):
+    """(peak in FLOP/s, its source) of the FP64 pipe: two FMAs per clock and SM at the largest SM
+    clock, unless the probe's chains got more.  (They get less: 1.10 of 1.26 TFLOP/s, where the
+    product kernel gets 1.13.)"""
+    pipe = n_sms * 4.0 * sm_max_mhz * 1e6 if n_sms and sm_max_mhz else 0.0
+    if pipe > probe:
+        return pipe, "FP64 pipe: 2 FMAs per clock on %d SMs at %.0f MHz" % (n_sms, sm_max_mhz)
+    return probe, "in-library FP64 probe (best of FMA and DMMA chains)"
 
 
 def measured_peaks():
@@ -852,6 +862,8 @@ def run_cq(args, rank, world, local_rank):
         n_launch, kern_ms, kern_flops, mma_flops = main["stats"]
         ms = main["ms"]
         achieved = kern_flops / (kern_ms * 1e-3) / 1e12 if kern_ms > 0 else None
+        n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
+        peak, peak_source = fp64_peak(peak_fp64, n_sms, main["clk"].get("sm_max_mhz"))
         line = {
             "metric": METRIC,
             "value": main["flops_all"] / (ms * 1e-3) / 1e9, "unit": "GFLOP/s", "n_gpus": world,
@@ -862,11 +874,11 @@ def run_cq(args, rank, world, local_rank):
             "config": bench_config(cell, args, world),
             "hotelling_resid": resid[-1] if resid else None,
             "roofline": {"bound": "alu", "kernel": "k_bsmm_f64_uniform",
-                         "achieved": achieved, "peak": peak_fp64 / 1e12, "unit": "TFLOP/s",
-                         "frac": (achieved / (peak_fp64 / 1e12)) if achieved else None,
+                         "achieved": achieved, "peak": peak / 1e12, "unit": "TFLOP/s",
+                         "frac": (achieved / (peak / 1e12)) if achieved else None,
                          "traffic": FP64_TRAFFIC_PER_LAUNCH if cell.n_atoms == 4096 else None,
                          "traffic_source": TRAFFIC_SOURCE,
-                         "peak_source": "in-library FP64 probe (best of FMA and DMMA chains)",
+                         "peak_source": peak_source, "probe": peak_fp64 / 1e12,
                          "launches": n_launch, "kernel_ms": kern_ms,
                          "kernel_share": kern_ms / ms if ms > 0 else None},
             "lnv": [{k: x[k] for k in ("energy", "n_elec", "gnorm", "alpha", "n_corr",
